@@ -23,6 +23,8 @@
 //  k_lines_tma  contiguous FP32 systems of 256 < N <= 4096 in one pass:
 //             whole systems staged in shared memory by bulk copies, one team
 //             of warps per system (trid_lines_tma.cuh).
+//  k_twist    FP64 systems of N <= 256, when there are many: Thomas from both
+//             ends, two threads per system (trid_twist.cuh).
 //  k_chunk_cluster  strided FP32 systems of 256 < N <= 4096 in one pass:
 //             chunks of 256 or 512 rows, one CTA each, joined by a chunk-level
 //             solve across a thread-block cluster (trid_chunked.cuh).
@@ -30,6 +32,7 @@
 #include "trid_strided.cuh"
 #include "trid_lines_tma.cuh"
 #include "trid_chunked.cuh"
+#include "trid_twist.cuh"
 #include "../../include/trid.h"
 #include "trid_internal.h"
 
@@ -451,12 +454,58 @@ static bool launch_chunk_cluster(const T *a, const T *b, const T *c, const T *d,
     }
 }
 
+// FP64 systems of up to 256 rows through k_twist, when there are enough of
+// them: its time does not fall below the latency of one system's two chains
+// (256 rows: 53 us strided, 65 us contiguous, for any number of systems up to
+// about 9700), where the tiled kernels take 0.0125 us (strided) and 0.012 us
+// (contiguous) per 256-row system, both in proportion to the rows: the times
+// cross at 4096 strided (53 against 51 us) and about 6000 contiguous systems
+// (6144 of 128 rows: 35 against 38 us).  At 65536 systems of 256 rows they
+// are 305 against 655 us (strided) and 381 against 596 us (contiguous).
+// Contiguous systems only when their halves are whole 32-byte vectors (with
+// scalar loads 378 us against 402 us at 43571 systems of 201 rows, and slower
+// than that at two warps per block), and not when accumulating (d' then
+// fills the shared memory: 711 us against 629 us; strided 534 against 678).
+// False, having launched nothing, when the tiled kernels are to be used.
+template <bool ACC, bool VEC, int WARPS>
+static bool launch_twist_form(const double *a, const double *b, const double *c, const double *d,
+                              double *out, const Lines &L, cudaStream_t st) {
+    const size_t smem = twist_smem(int(L.n), VEC, ACC, WARPS);
+    auto kern = k_twist<ACC, VEC, WARPS>;
+    if (kernel_blocks_per_sm(reinterpret_cast<const void *>(kern), 32 * WARPS, smem) < 1)
+        return false;
+    const int64_t blocks = (L.nsys + WARPS * TW_SYS - 1) / (WARPS * TW_SYS);
+    if (blocks >= (int64_t(1) << 31)) return false;
+    kern<<<dim3(unsigned(blocks)), 32 * WARPS, smem, st>>>(a, b, c, d, out, L);
+    return launch_ok();
+}
+
+template <typename T>
+static bool launch_twist(const T *a, const T *b, const T *c, const T *d, T *out, int acc,
+                         const Lines &L, cudaStream_t st) {
+    if constexpr (!std::is_same<T, double>::value) {
+        return false;
+    } else {
+        if (!b || L.n > MAX_SINGLE_PASS || !strided_offsets_fit(L)) return false;
+        if (L.stride == 1) {
+            auto al32 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; };
+            return L.nsys >= 6144 && !acc && L.n % 4 == 0 && al32(a) && al32(b) && al32(c) &&
+                   al32(d) && al32(out) &&
+                   launch_twist_form<false, true, 2>(a, b, c, d, out, L, st);
+        }
+        if (L.nsys < 4608) return false;
+        return acc ? launch_twist_form<true, false, 1>(a, b, c, d, out, L, st)
+                   : launch_twist_form<false, false, 1>(a, b, c, d, out, L, st);
+    }
+}
+
 template <typename T>
 static trid_status solve_lines(const T *a, const T *b, const T *c, const T *d, T *out, int acc,
                                const Lines &L, char *ws, size_t ws_bytes, cudaStream_t st) {
     if (L.nsys == 0 || L.n == 0) return TRID_OK;
     const bool contig = (L.stride == 1);
     if (L.n <= MAX_SINGLE_PASS) {
+        if (launch_twist<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
         const int G = pow2_at_least((L.n + TILE_M - 1) / TILE_M);
         if (contig) {
             const int vec_ok = is_aligned16(a) && is_aligned16(c) && is_aligned16(d) &&
