@@ -3,20 +3,24 @@
 // Section 4 and the chained-iteration (temporal) pipelining of the 2D ADI
 // design).
 //
-// When one mesh and its right-hand side fit in one block's shared memory, a
-// block loads the mesh once, runs all nsteps steps in shared memory and writes
-// it back: per step the 5-point / 7-point RHS, then one thread per line runs
-// the Thomas sweeps of each axis with the constant operator's pivots factored
-// once on the host, the last axis adding its result into u.  Rows are padded
-// to an odd stride, so the threads of a warp (one line each) hit distinct
-// banks on every axis.  Larger 3D meshes whose extents suit the two-pass
-// schedule run stacked along z through its kernels (each mesh keeps its own
-// boundary planes); the rest go through adi_step one mesh at a time.
+// 2D meshes that fit one block's shared memory, up to 160 (FP64: 128) nodes
+// along an axis, run every step of the call on chip in k_adi_plane
+// (trid_adi_plane.cuh).  3D meshes (and the few 2D ones beyond that) whose
+// field and right-hand side fit do so in k_adi_fused: a block loads the mesh
+// once, runs all nsteps steps in shared memory and writes it back: per step the
+// 5-point / 7-point RHS, then one thread per line runs the Thomas sweeps of
+// each axis with the constant operator's pivots factored once on the host, the
+// last axis adding its result into u.  Rows are padded to an odd stride, so
+// the threads of a warp (one line each) hit distinct banks on every axis.
+// Larger 3D meshes whose extents suit the two-pass schedule run stacked along
+// z through its kernels (each mesh keeps its own boundary planes); the rest go
+// through adi_step one mesh at a time.
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
 #include "../../include/trid.h"
+#include "trid_adi_plane.cuh"
 #include "trid_internal.h"
 
 namespace trid {
@@ -209,9 +213,78 @@ static bool ba_plan(const int64_t *n3, int ndim, size_t esz, BaPlan &pl) {
     return true;
 }
 
+// 2D meshes through k_adi_plane.  Warps per block: a phase walks its groups of
+// 16 lines, and a mesh occupies its warps for the walks of both phases; the
+// number with the least (rounds of blocks) x (rows walked), of equal ones the
+// largest (128 x 32, 2000 meshes, 40 steps, an earlier form: 8 warps 2014 us,
+// 2 warps 1108 us).  False, having launched nothing, when the mesh does not fit.
+template <typename T, int HX, int HY>
+static bool plane_run_h(T *u, int64_t nbatch, int nx, int ny, double lam, int nsteps,
+                        cudaStream_t st) {
+    const int hx = (nx + 1) / 2, hy = (ny + 1) / 2;
+    const size_t smem = size_t(plane_layout<T>(plane_pitch<T>(HX), hy).total) * sizeof(T);
+    const DeviceInfo *di = device_info();
+    auto kern = k_adi_plane<T, HX, HY>;
+    if (!di || smem > size_t(di->max_smem_optin)) return false;
+    const int gx = plane_groups(ny), gy = plane_groups(nx);
+    int threads = 0;
+    int64_t grid = 0, best = 0;
+    for (int w = 1; w <= (gx > gy ? gx : gy); ++w) {
+        const int per_sm =
+            kernel_blocks_per_sm(reinterpret_cast<const void *>(kern), 32 * w, smem);
+        if (per_sm < 1) continue;
+        const int64_t slots = int64_t(di->sm_count) * per_sm;
+        const int64_t rounds = (nbatch + slots - 1) / slots;
+        const int64_t cost = rounds * ((gx + w - 1) / w * hx + (gy + w - 1) / w * hy);
+        if (threads == 0 || cost <= best) {
+            best = cost;
+            threads = 32 * w;
+            grid = nbatch < slots ? nbatch : slots;
+        }
+    }
+    if (threads == 0) return false;
+    PlaneTabs<T, HX, HY> t;
+    plane_axis<T, HX>(t.fx, t.gx, t.kx, nx, lam, lam);
+    plane_axis<T, HY>(t.fy, t.gy, t.ky, ny, lam, 1.0);
+    kern<<<dim3(unsigned(grid)), threads, smem, st>>>(u, nbatch, nx, ny, nsteps, t);
+    return launch_ok();
+}
+
+template <typename T, int HX>
+static bool plane_run_x(T *u, int64_t nbatch, int nx, int ny, double lam, int nsteps,
+                        cudaStream_t st) {
+    switch ((ny + 2 * PL_STEP - 1) / (2 * PL_STEP)) {
+        case 1: return plane_run_h<T, HX, 16>(u, nbatch, nx, ny, lam, nsteps, st);
+        case 2: return plane_run_h<T, HX, 32>(u, nbatch, nx, ny, lam, nsteps, st);
+        case 3: return plane_run_h<T, HX, 48>(u, nbatch, nx, ny, lam, nsteps, st);
+        case 4: return plane_run_h<T, HX, 64>(u, nbatch, nx, ny, lam, nsteps, st);
+        case 5:   // FP64 lines of 80 leave no registers
+            if constexpr (sizeof(T) == 4)
+                return plane_run_h<T, HX, 80>(u, nbatch, nx, ny, lam, nsteps, st);
+        default: return false;
+    }
+}
+
+template <typename T>
+static bool plane_run(T *u, int64_t nbatch, int nx, int ny, double lam, int nsteps,
+                      cudaStream_t st) {
+    switch ((nx + 2 * PL_STEP - 1) / (2 * PL_STEP)) {
+        case 1: return plane_run_x<T, 16>(u, nbatch, nx, ny, lam, nsteps, st);
+        case 2: return plane_run_x<T, 32>(u, nbatch, nx, ny, lam, nsteps, st);
+        case 3: return plane_run_x<T, 48>(u, nbatch, nx, ny, lam, nsteps, st);
+        case 4: return plane_run_x<T, 64>(u, nbatch, nx, ny, lam, nsteps, st);
+        case 5:
+            if constexpr (sizeof(T) == 4)
+                return plane_run_x<T, 80>(u, nbatch, nx, ny, lam, nsteps, st);
+        default: return false;
+    }
+}
+
 template <typename T>
 static trid_status ba_run(T *u, int64_t nbatch, const int64_t *n3, int ndim, double lam,
                           int nsteps, const BaPlan &pl, cudaStream_t st) {
+    if (ndim == 2 && plane_run<T>(u, nbatch, int(n3[0]), int(n3[1]), lam, nsteps, st))
+        return TRID_OK;
     BTabs<T> tabs;
     for (int k = 0; k < 3; ++k) baxis_fill<T>(tabs.ax[k], int(n3[k]), lam);
     const void *kern = ndim == 2 ? reinterpret_cast<const void *>(k_adi_fused<T, 2>)
