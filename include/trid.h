@@ -340,15 +340,17 @@ trid_status trid_varlen_autotune(const void *a, const void *b, const void *c, co
  * 2D / 3D workloads of Section 4).  u holds nbatch meshes of dims[0] x ...
  * x dims[ndim-1] points (ndim 2 or 3, every extent 3..256), mesh b starting
  * at element b * (product of dims), each column-major (x contiguous); every
- * mesh advances by nsteps steps exactly as with adi_step.  When a mesh and its
- * right-hand side fit one block's shared memory, all nsteps steps run in one
- * kernel with the mesh resident on chip (read and written once per call);
- * otherwise 3D meshes whose extents suit the two-pass 3D schedule (all
- * multiples of 16, z >= 32) run stacked along z through its kernels, and the
- * rest go through adi_step one after another.  `workspace` (256-byte
- * aligned) must hold adi_batched_workspace_bytes(nbatch, dims, ndim, dtype)
- * bytes (0 in the resident case, where workspace may be NULL).  Errors as
- * adi_step; asynchronous on `stream`.
+ * mesh advances by nsteps steps as with adi_step.  When a mesh and its
+ * right-hand side fit one block's shared memory, all nsteps steps can run in
+ * one kernel with the mesh resident on chip (read and written once per call);
+ * 3D meshes run stacked along z through the kernels of the 3D step, and the
+ * rest go through adi_step one after another.  `workspace` (256-byte aligned)
+ * should hold adi_batched_workspace_bytes(nbatch, dims, ndim, dtype) bytes.
+ * It must do so when every extent is a multiple of 16 and z is at least 32;
+ * other 3D meshes are also stepped with less, as many at a time as it holds:
+ * the least is the scratch of one mesh (adi_workspace_bytes), and none
+ * (workspace NULL) where a mesh can be resident on chip.  Errors as adi_step;
+ * asynchronous on `stream`.
  */
 size_t adi_batched_workspace_bytes(int64_t nbatch, const int64_t *dims, int ndim,
                                    trid_dtype dtype);

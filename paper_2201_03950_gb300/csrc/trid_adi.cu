@@ -12,6 +12,10 @@
 //     below 1/16 ulp within 8 rows): k_adi_xyw (stencil + x solve + windowed
 //     y solve per plane cluster, writes e = Z u + Y^{-1} X^{-1} d) and k_adi_zw
 //     (windowed z solve, u = Z^{-1} e); 4 mesh words per point.
+//   whole planes (trid_adi_planes.cuh, planes that fit an SM's shared memory
+//     three times, up to 160 nodes an axis; any lambda, FP32 and FP64): the
+//     explicit part and the x and y solves of a plane in one block, then the
+//     z lines in registers; 5 words.
 //   two-pass (trid_adi_2pass.cuh, extents multiples of 16): k_adi_xy and
 //     k_adi_z_ysub, the y solve split by the Section 3.1 tiling across them.
 //   general (any extents <= 256): stencil + x solve (k_adi_x_static or
@@ -667,6 +671,33 @@ static trid_status adi_dims(const int64_t *dims, int ndim, int64_t (&n3)[3], int
     return TRID_OK;
 }
 
+// Planes of up to 32 x 32 points: the whole-plane schedule before the windowed
+// one (72 meshes of 32^3: 13.6 against 15.5 us a step, one mesh 5.4 against
+// 7.4; 80 x 32 x 32, 72 meshes: 30.0 against 24.6).
+static bool adi_small_planes(const int64_t *n3) { return n3[0] <= 32 && n3[1] <= 32; }
+
+// nb meshes stacked along z through the whole-plane schedule, where it is the
+// faster one: not for few, long z lines (pass B has a thread per half line;
+// 31 x 40 x 200, one mesh: 17.8 against 14.6 us a step), nor in FP64 for
+// planes that leave half of the SMs without one when the two-pass schedule,
+// which cuts planes into tiles, can run (64^3, one mesh: 43.6 against 39.1;
+// 80^3 43.4 against 67.8).  `taken` is false, and nothing launched, otherwise.
+trid_status adi3_planes_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
+                            trid_dtype dtype, void *ws, cudaStream_t st, bool &taken) {
+    taken = false;
+    const DeviceInfo *di = device_info();
+    if (!di || n3[2] < 3) return TRID_OK;
+    if (n3[2] > 160 && n3[0] * n3[1] * nb < 2048) return TRID_OK;
+    if (dtype == TRID_F64 && adi2_eligible(n3, 3) && n3[0] * n3[1] >= 4096 &&
+        nb * (n3[2] - 2) * 2 < di->sm_count)
+        return TRID_OK;
+    if (dtype == TRID_F32)
+        return adi_planes_run(static_cast<float *>(u), static_cast<float *>(ws), n3, nb, lam,
+                              nsteps, st, taken);
+    return adi_planes_run(static_cast<double *>(u), static_cast<double *>(ws), n3, nb, lam, nsteps,
+                          st, taken);
+}
+
 // Batches of 3D meshes stacked along z (each mesh keeps its own boundary
 // planes), through the two-pass schedule; used by adi_step_batched.
 bool adi3_batch_eligible(const int64_t *n3, int ndim) { return adi2_eligible(n3, ndim); }
@@ -681,12 +712,13 @@ trid_status adi3_batch_run(void *u, int64_t nb, const int64_t *n3, double lam, i
     if (!ws || ws_bytes < adi3_batch_ws_bytes(n3, esz, nb)) return TRID_ERR_ALLOC;
     if ((reinterpret_cast<uintptr_t>(ws) % 256) != 0) return TRID_ERR_MISALIGNED;
     if (!is_aligned16(u)) return TRID_ERR_MISALIGNED;
-    if (dtype == TRID_F32) {
-        bool taken = false;
-        const trid_status s = adi_run_window(static_cast<float *>(u), n3, lam, nsteps,
-                                             static_cast<char *>(ws), st, nb, taken);
-        if (taken || s != TRID_OK) return s;
-    }
+    bool taken = false;
+    trid_status s = TRID_OK;
+    if (dtype == TRID_F32 && !adi_small_planes(n3))
+        s = adi_run_window(static_cast<float *>(u), n3, lam, nsteps, static_cast<char *>(ws), st,
+                           nb, taken);
+    if (!taken && s == TRID_OK) s = adi3_planes_run(u, nb, n3, lam, nsteps, dtype, ws, st, taken);
+    if (taken || s != TRID_OK) return s;
     if (dtype == TRID_F32)
         return adi_run_2pass<float>(static_cast<float *>(u), n3, float(lam), nsteps,
                                     static_cast<char *>(ws), st, nb);
@@ -729,10 +761,13 @@ extern "C" trid_status adi_step(void *u, const int64_t *dims, int ndim, double l
     }
     if (nsteps == 0) return TRID_OK;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (ndim == 3 && dtype == TRID_F32) {
+    if (ndim == 3) {
         bool taken = false;
-        s = adi_run_window(static_cast<float *>(u), n3, lambda, nsteps,
-                           static_cast<char *>(workspace), st, 1, taken);
+        if (dtype == TRID_F32 && !adi_small_planes(n3))
+            s = adi_run_window(static_cast<float *>(u), n3, lambda, nsteps,
+                               static_cast<char *>(workspace), st, 1, taken);
+        if (!taken && s == TRID_OK)
+            s = adi3_planes_run(u, 1, n3, lambda, nsteps, dtype, workspace, st, taken);
         if (taken || s != TRID_OK) return s;
     }
     if (adi2_eligible(n3, ndim) && is_aligned16(u)) {

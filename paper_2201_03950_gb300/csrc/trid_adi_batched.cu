@@ -5,22 +5,20 @@
 //
 // 2D meshes that fit one block's shared memory, up to 160 (FP64: 128) nodes
 // along an axis, run every step of the call on chip in k_adi_plane
-// (trid_adi_plane.cuh).  3D meshes (and the few 2D ones beyond that) whose
-// field and right-hand side fit do so in k_adi_fused: a block loads the mesh
-// once, runs all nsteps steps in shared memory and writes it back: per step the
-// 5-point / 7-point RHS, then one thread per line runs the Thomas sweeps of
-// each axis with the constant operator's pivots factored once on the host, the
-// last axis adding its result into u.  Rows are padded to an odd stride, so
-// the threads of a warp (one line each) hit distinct banks on every axis.
-// Larger 3D meshes whose extents suit the two-pass schedule run stacked along
-// z through its kernels (each mesh keeps its own boundary planes); the rest go
-// through adi_step one mesh at a time.
+// (trid_adi_plane.cuh).  Small 3D meshes (and the few 2D ones beyond that) do
+// so in k_adi_fused: a block loads the mesh once, runs all nsteps steps in
+// shared memory and writes it back: per step the 5-point / 7-point RHS, then
+// one thread per line runs the Thomas sweeps of each axis with the constant
+// operator's pivots factored once on the host, the last axis adding its result
+// into u.  Rows are padded to an odd stride, so the threads of a warp (one line
+// each) hit distinct banks on every axis.  The other 3D meshes run stacked
+// along z through the windowed, whole-plane or two-pass kernels (each mesh keeps
+// its own boundary planes), those that suit none one mesh at a time.
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
 #include "../../include/trid.h"
-#include "trid_adi_plane.cuh"
 #include "trid_internal.h"
 
 namespace trid {
@@ -213,78 +211,15 @@ static bool ba_plan(const int64_t *n3, int ndim, size_t esz, BaPlan &pl) {
     return true;
 }
 
-// 2D meshes through k_adi_plane.  Warps per block: a phase walks its groups of
-// 16 lines, and a mesh occupies its warps for the walks of both phases; the
-// number with the least (rounds of blocks) x (rows walked), of equal ones the
-// largest (128 x 32, 2000 meshes, 40 steps, an earlier form: 8 warps 2014 us,
-// 2 warps 1108 us).  False, having launched nothing, when the mesh does not fit.
-template <typename T, int HX, int HY>
-static bool plane_run_h(T *u, int64_t nbatch, int nx, int ny, double lam, int nsteps,
-                        cudaStream_t st) {
-    const int hx = (nx + 1) / 2, hy = (ny + 1) / 2;
-    const size_t smem = size_t(plane_layout<T>(plane_pitch<T>(HX), hy).total) * sizeof(T);
-    const DeviceInfo *di = device_info();
-    auto kern = k_adi_plane<T, HX, HY>;
-    if (!di || smem > size_t(di->max_smem_optin)) return false;
-    const int gx = plane_groups(ny), gy = plane_groups(nx);
-    int threads = 0;
-    int64_t grid = 0, best = 0;
-    for (int w = 1; w <= (gx > gy ? gx : gy); ++w) {
-        const int per_sm =
-            kernel_blocks_per_sm(reinterpret_cast<const void *>(kern), 32 * w, smem);
-        if (per_sm < 1) continue;
-        const int64_t slots = int64_t(di->sm_count) * per_sm;
-        const int64_t rounds = (nbatch + slots - 1) / slots;
-        const int64_t cost = rounds * ((gx + w - 1) / w * hx + (gy + w - 1) / w * hy);
-        if (threads == 0 || cost <= best) {
-            best = cost;
-            threads = 32 * w;
-            grid = nbatch < slots ? nbatch : slots;
-        }
-    }
-    if (threads == 0) return false;
-    PlaneTabs<T, HX, HY> t;
-    plane_axis<T, HX>(t.fx, t.gx, t.kx, nx, lam, lam);
-    plane_axis<T, HY>(t.fy, t.gy, t.ky, ny, lam, 1.0);
-    kern<<<dim3(unsigned(grid)), threads, smem, st>>>(u, nbatch, nx, ny, nsteps, t);
-    return launch_ok();
-}
-
-template <typename T, int HX>
-static bool plane_run_x(T *u, int64_t nbatch, int nx, int ny, double lam, int nsteps,
-                        cudaStream_t st) {
-    switch ((ny + 2 * PL_STEP - 1) / (2 * PL_STEP)) {
-        case 1: return plane_run_h<T, HX, 16>(u, nbatch, nx, ny, lam, nsteps, st);
-        case 2: return plane_run_h<T, HX, 32>(u, nbatch, nx, ny, lam, nsteps, st);
-        case 3: return plane_run_h<T, HX, 48>(u, nbatch, nx, ny, lam, nsteps, st);
-        case 4: return plane_run_h<T, HX, 64>(u, nbatch, nx, ny, lam, nsteps, st);
-        case 5:   // FP64 lines of 80 leave no registers
-            if constexpr (sizeof(T) == 4)
-                return plane_run_h<T, HX, 80>(u, nbatch, nx, ny, lam, nsteps, st);
-        default: return false;
-    }
-}
-
-template <typename T>
-static bool plane_run(T *u, int64_t nbatch, int nx, int ny, double lam, int nsteps,
-                      cudaStream_t st) {
-    switch ((nx + 2 * PL_STEP - 1) / (2 * PL_STEP)) {
-        case 1: return plane_run_x<T, 16>(u, nbatch, nx, ny, lam, nsteps, st);
-        case 2: return plane_run_x<T, 32>(u, nbatch, nx, ny, lam, nsteps, st);
-        case 3: return plane_run_x<T, 48>(u, nbatch, nx, ny, lam, nsteps, st);
-        case 4: return plane_run_x<T, 64>(u, nbatch, nx, ny, lam, nsteps, st);
-        case 5:
-            if constexpr (sizeof(T) == 4)
-                return plane_run_x<T, 80>(u, nbatch, nx, ny, lam, nsteps, st);
-        default: return false;
-    }
-}
-
 template <typename T>
 static trid_status ba_run(T *u, int64_t nbatch, const int64_t *n3, int ndim, double lam,
                           int nsteps, const BaPlan &pl, cudaStream_t st) {
-    if (ndim == 2 && plane_run<T>(u, nbatch, int(n3[0]), int(n3[1]), lam, nsteps, st))
-        return TRID_OK;
+    if (ndim == 2) {
+        bool taken = false;
+        const trid_status s =
+            adi_plane_run(u, nbatch, int(n3[0]), int(n3[1]), lam, nsteps, st, taken);
+        if (taken) return s;
+    }
     BTabs<T> tabs;
     for (int k = 0; k < 3; ++k) baxis_fill<T>(tabs.ax[k], int(n3[k]), lam);
     const void *kern = ndim == 2 ? reinterpret_cast<const void *>(k_adi_fused<T, 2>)
@@ -307,6 +242,22 @@ static trid_status ba_run(T *u, int64_t nbatch, const int64_t *n3, int ndim, dou
 
 using namespace trid;
 
+// 3D meshes small enough for k_adi_fused that the whole-plane kernels step
+// faster, given scratch: in FP32 from 2048 points on (24^3: 24 meshes 18.5 ->
+// 9.7 us a step, 1000 meshes 128 -> 78; 16^3, 72 meshes: 12.0 -> 7.7; 8^3, 1000
+// meshes: 9.8 against 11.2), but not many meshes much longer along x than along
+// y, whose short columns fill few lanes (64 x 16 x 16, 1000 meshes: 76 against
+// 88; 67 x 16 x 17, 8 meshes: 14.9 -> 7.1).  In FP64 k_adi_fused is as fast or
+// faster (16^3, 72 meshes: 30 against 38; 8^3, 1000: 28 against 47).
+static bool ba_planes_first(const int64_t *n3, size_t esz, int64_t nb) {
+    return esz == 4 && n3[0] * n3[1] * n3[2] >= 2048 && (nb <= 300 || n3[0] <= 2 * n3[1]);
+}
+
+// Scratch of nb meshes stacked through the whole-plane schedule.
+static size_t ba_stack_bytes(const int64_t *n3, size_t esz, int64_t nb) {
+    return (size_t(n3[0] * n3[1] * n3[2]) * esz * size_t(nb) + 255) / 256 * 256;
+}
+
 static trid_status ba_dims(const int64_t *dims, int ndim, int64_t (&n3)[3]) {
     if (!dims || ndim < 2 || ndim > 3) return TRID_ERR_INVALID_ARG;
     n3[0] = n3[1] = n3[2] = 1;
@@ -327,9 +278,12 @@ extern "C" size_t adi_batched_workspace_bytes(int64_t nbatch, const int64_t *dim
     const size_t esz = dtype == TRID_F32 ? 4 : 8;
     BaPlan pl;
     if (!ba_plan(n3, ndim, esz, pl)) return 0;
-    if (pl.fused || nbatch == 0) return 0;
-    if (adi3_batch_eligible(n3, ndim)) return adi3_batch_ws_bytes(n3, esz, nbatch);
-    return adi_workspace_bytes(dims, ndim, dtype);
+    if (nbatch == 0 || (pl.fused && ndim == 2)) return 0;
+    if (!pl.fused && adi3_batch_eligible(n3, ndim)) return adi3_batch_ws_bytes(n3, esz, nbatch);
+    const size_t one = pl.fused ? 0 : adi_workspace_bytes(dims, ndim, dtype);
+    const size_t all = ndim == 3 && (!pl.fused || ba_planes_first(n3, esz, nbatch))
+                           ? ba_stack_bytes(n3, esz, nbatch) : 0;
+    return one > all ? one : all;
 }
 
 extern "C" trid_status adi_step_batched(void *u, int64_t nbatch, const int64_t *dims, int ndim,
@@ -349,20 +303,43 @@ extern "C" trid_status adi_step_batched(void *u, int64_t nbatch, const int64_t *
     BaPlan pl;
     if (!ba_plan(n3, ndim, esz, pl)) return TRID_ERR_CUDA;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (pl.fused) {
-        if (dtype == TRID_F32)
-            return ba_run<float>(static_cast<float *>(u), nbatch, n3, ndim, lambda, nsteps, pl, st);
-        return ba_run<double>(static_cast<double *>(u), nbatch, n3, ndim, lambda, nsteps, pl, st);
-    }
-    // 3D meshes stacked along z through the two-pass kernels (boundary planes
-    // per mesh), when the extents allow it
-    if (adi3_batch_eligible(n3, ndim) && n3[2] * nbatch <= 65535)
-        return adi3_batch_run(u, nbatch, n3, lambda, nsteps, dtype, workspace, workspace_bytes, st);
-    // otherwise one mesh at a time through the single-mesh path
+    // 3D meshes stacked along z through the windowed, whole-plane or two-pass
+    // kernels (boundary planes per mesh)
     const size_t mesh = size_t(n3[0] * n3[1] * n3[2]) * esz;
-    for (int64_t b = 0; b < nbatch; ++b) {
-        s = adi_step(static_cast<char *>(u) + b * mesh, dims, ndim, lambda, nsteps, dtype,
-                     workspace, workspace_bytes, stream);
+    if (!pl.fused && adi3_batch_eligible(n3, ndim) && n3[2] * nbatch <= 65535)
+        return adi3_batch_run(u, nbatch, n3, lambda, nsteps, dtype, workspace, workspace_bytes, st);
+    // other 3D meshes through the whole-plane kernels, as many at a time as the
+    // scratch holds
+    int64_t done = 0;
+    char *pu = static_cast<char *>(u);
+    if (ndim == 3 && workspace && (reinterpret_cast<uintptr_t>(workspace) % 256) == 0 &&
+        (!pl.fused || ba_planes_first(n3, esz, nbatch))) {
+        const char *pw = static_cast<const char *>(workspace);
+        const bool apart = pu >= pw + workspace_bytes || pw >= pu + mesh * size_t(nbatch);
+        int64_t group = apart ? int64_t(workspace_bytes / mesh) : 0;
+        if (group > 65535) group = 65535;
+        bool taken = group > 0;
+        while (taken && done < nbatch) {
+            const int64_t nb = nbatch - done < group ? nbatch - done : group;
+            s = adi3_planes_run(pu + size_t(done) * mesh, nb, n3, lambda, nsteps, dtype, workspace,
+                                st, taken);
+            if (s != TRID_OK) return s;
+            if (taken) done += nb;
+        }
+        if (done == nbatch) return TRID_OK;
+    }
+    if (pl.fused) {
+        pu += size_t(done) * mesh;
+        if (dtype == TRID_F32)
+            return ba_run<float>(reinterpret_cast<float *>(pu), nbatch - done, n3, ndim, lambda,
+                                 nsteps, pl, st);
+        return ba_run<double>(reinterpret_cast<double *>(pu), nbatch - done, n3, ndim, lambda,
+                              nsteps, pl, st);
+    }
+    // otherwise one mesh at a time through the single-mesh path
+    for (; done < nbatch; ++done) {
+        s = adi_step(pu + size_t(done) * mesh, dims, ndim, lambda, nsteps, dtype, workspace,
+                     workspace_bytes, stream);
         if (s != TRID_OK) return s;
     }
     return TRID_OK;

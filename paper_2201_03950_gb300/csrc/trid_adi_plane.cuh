@@ -51,10 +51,33 @@ struct PlaneTabs {
     T kx, ky;   // 1 / (1 - G G') of the middle
 };
 
-// Half lines are held in HX and HY registers, multiples of 16 that exceed the
-// half line by less than 16: only the first 16 can be empty.  The row pitch
-// follows from HX, so that every address of a sweep is a constant offset.
+// Half lines are held in HX and HY registers, of the sizes below: the smallest
+// that holds the half line, which leaves fewer than 16 empty, so that only the
+// first 16 need be looked at.  The row pitch follows from HX, so that every
+// address of a sweep is a constant offset.
 constexpr int PL_STEP = 16;
+inline int plane_size(int n) {   // of a line of n nodes; 0: too long
+    const int h = (n + 1) / 2;
+    return h <= 16 ? 16 : h <= 48 ? (h + 7) / 8 * 8 : h <= 80 ? (h + 15) / 16 * 16 : 0;
+}
+// Calls f with the size as a compile-time constant; FP64 lines of 80 leave no
+// registers.
+template <int H> struct PlaneSize { static constexpr int value = H; };
+template <typename T, typename F>
+inline bool plane_dispatch(int n, F &&f) {
+    switch (plane_size(n)) {
+        case 16: return f(PlaneSize<16>());
+        case 24: return f(PlaneSize<24>());
+        case 32: return f(PlaneSize<32>());
+        case 40: return f(PlaneSize<40>());
+        case 48: return f(PlaneSize<48>());
+        case 64: return f(PlaneSize<64>());
+        case 80:
+            if constexpr (sizeof(T) == 4) return f(PlaneSize<80>());
+            return false;
+        default: return false;
+    }
+}
 template <typename T>
 __host__ __device__ constexpr int plane_pitch(int HX) { return 2 * HX + 16 / int(sizeof(T)); }
 
@@ -112,13 +135,17 @@ constexpr int plane_min_blocks(int HX, int HY, int esz) {
     const int nb = 16384 / (32 * words) * 4 / plane_max_warps(HX, HY);
     return nb < 1 ? 1 : nb;
 }
+// The warps per SM that this leaves room for.
+constexpr int plane_sm_warps(int HX, int HY, int esz) {
+    return plane_min_blocks(HX, HY, esz) * plane_max_warps(HX, HY);
+}
 
 template <typename T, int HX, int HY>
 __global__ void __launch_bounds__(32 * plane_max_warps(HX, HY),
                                   plane_min_blocks(HX, HY, sizeof(T)))
 k_adi_plane(T *__restrict__ ug, int64_t nbatch, int nx, int ny, int nsteps,
             const __grid_constant__ PlaneTabs<T, HX, HY> t) {
-    static_assert(HX % PL_STEP == 0 && HY % PL_STEP == 0, "half lines in whole steps");
+    static_assert(HX % 4 == 0 && HY % 4 == 0, "whole groups of four");
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int CX = HX / 4, CY = HY / 4, CG = PL_STEP / 4;  // groups of 4; those that may be empty
     constexpr int p = plane_pitch<T>(HX);
@@ -274,6 +301,35 @@ inline void plane_axis(T (&f)[H], T (&g)[H], T &k, int n, double lam, double sca
         g[q] = T(gd[q]);
     }
     k = T(1.0 / (1.0 - gd[H - 1] * gd[H - 1 - (n & 1)]));
+}
+
+// Host: warps per block for `items` planes.  A phase walks its groups of 16
+// lines and a plane occupies its warps for the walks of both phases (and for
+// loading `load_points` points); the number with the least (rounds of blocks)
+// x (rows walked), of equal ones the largest.  128 x 32 planes, 2000 meshes,
+// 40 steps (an earlier form of k_adi_plane): 8 warps 2014 us, 2 warps 1108 us.
+// warps_per_sm: what the registers allow.
+inline int plane_pick_warps(int64_t items, int nx, int ny, int load_points, size_t smem,
+                            size_t smem_per_sm, int sm_count, int warps_per_sm, int max_warps) {
+    const int gx = plane_groups(ny), gy = plane_groups(nx);
+    const int hx = (nx + 1) / 2, hy = (ny + 1) / 2;
+    int pick = 1;
+    int64_t best = -1;
+    for (int w = 1; w <= (gx > gy ? gx : gy) && w <= max_warps; ++w) {
+        int64_t per_sm = int64_t(smem_per_sm / (smem + 1024));
+        if (per_sm > warps_per_sm / w) per_sm = warps_per_sm / w;
+        if (per_sm > 32) per_sm = 32;
+        if (per_sm < 1) per_sm = 1;
+        const int64_t slots = per_sm * sm_count;
+        const int64_t rounds = (items + slots - 1) / slots;
+        const int64_t walk = (gx + w - 1) / w * hx + (gy + w - 1) / w * hy;
+        const int64_t cost = rounds * (walk + load_points / (32 * w));
+        if (best < 0 || cost <= best) {
+            best = cost;
+            pick = w;
+        }
+    }
+    return pick;
 }
 
 }  // namespace trid

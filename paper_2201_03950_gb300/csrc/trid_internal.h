@@ -67,11 +67,33 @@ trid_status solve_with_scratch(const void *a, const void *b, const void *c, void
 // trid_get_device_status); kernels that run bounded waits record failures there.
 int *device_status_word();
 
-// 3D ADI on a batch of meshes stacked along z (two-pass schedule).
+// 3D ADI on nb meshes stacked along z through the whole-plane schedule, where it
+// is the fastest one (else `taken` is false and nothing is launched); ws holds
+// nb meshes.
+trid_status adi3_planes_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
+                            trid_dtype dtype, void *ws, cudaStream_t st, bool &taken);
+
+// 3D ADI on a batch of meshes stacked along z (windowed, whole-plane and
+// two-pass schedules).
 bool adi3_batch_eligible(const int64_t *n3, int ndim);
 size_t adi3_batch_ws_bytes(const int64_t *n3, size_t esz, int64_t nb);
 trid_status adi3_batch_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
                            trid_dtype dtype, void *ws, size_t ws_bytes, cudaStream_t st);
+
+// nsteps 2D ADI steps of nbatch meshes, each mesh on chip for all of them;
+// `taken` is false (nothing launched) when a mesh does not fit.
+trid_status adi_plane_run(float *u, int64_t nbatch, int nx, int ny, double lam, int nsteps,
+                          cudaStream_t st, bool &taken);
+trid_status adi_plane_run(double *u, int64_t nbatch, int nx, int ny, double lam, int nsteps,
+                          cudaStream_t st, bool &taken);
+
+// nsteps 3D ADI steps of nb meshes stacked along z through the whole-plane
+// kernels; w is a scratch array of the meshes' size.  `taken` is false (nothing
+// launched) when the extents do not suit them.
+trid_status adi_planes_run(float *u, float *w, const int64_t *n3, int64_t nb, double lam,
+                           int nsteps, cudaStream_t st, bool &taken);
+trid_status adi_planes_run(double *u, double *w, const int64_t *n3, int64_t nb, double lam,
+                           int nsteps, cudaStream_t st, bool &taken);
 
 // Allocation-free entry point's fixed array: looks its device address up on
 // the current device (true on success), and forgets the cached address of
