@@ -8,6 +8,7 @@ CPU fallback: if the library is missing or fails to load, every call raises.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 import threading
 
@@ -41,6 +42,8 @@ def lib_path() -> str:
 def load(path: str | None = None):
     """Load libtrid.so (built in-tree by ``build.build()``); raise if absent."""
     global _lib
+    if _lib is not None and path is None:
+        return _lib
     with _lock:
         if _lib is None or path is not None:
             p = path or lib_path()
@@ -92,9 +95,25 @@ def _bind(L):
         fn.restype = res
 
 
+_DIMS_CACHE: dict = {}
+_DIMS_CACHE_MAX = 256
+
+
+def _mesh(dims):
+    """(C array of the extents, their number, their product), kept by value: the
+    array is only read by the library."""
+    key = tuple(map(int, dims))
+    hit = _DIMS_CACHE.get(key)
+    if hit is None:
+        hit = (ctypes.c_int64 * max(len(key), 1))(*key), len(key), math.prod(key)
+        if len(_DIMS_CACHE) >= _DIMS_CACHE_MAX:
+            _DIMS_CACHE.clear()
+        _DIMS_CACHE[key] = hit
+    return hit
+
+
 def _dims(dims):
-    n = len(dims)
-    return (ctypes.c_int64 * max(n, 1))(*[int(v) for v in dims]), n
+    return _mesh(dims)[:2]
 
 
 def _dtype(t) -> int:
@@ -108,36 +127,37 @@ def _dtype(t) -> int:
 
 def _stream(stream):
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if torch.cuda.is_initialized():
+        # the current stream's handle without a Stream object around it (3 us)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _check_tensors(ts, dtype_ref, numel):
+    dtype = dtype_ref.dtype
     for t in ts:
         if t is None:
             continue
         if not t.is_cuda:
             raise ValueError("tensors must be CUDA tensors")
-        if t.dtype != dtype_ref.dtype:
+        if t.dtype is not dtype:
             raise TypeError("all arrays must share one dtype")
-        if not t.is_contiguous() or t.numel() != numel:
+        if t.numel() != numel or not t.is_contiguous():
             raise ValueError(f"arrays must be contiguous with {numel} elements")
 
 
 def solve(a, b, c, d, dims, solve_dim: int, u=None, workspace=None, stream=None):
     """Batched solve along ``solve_dim`` of a column-major mesh ``dims``
     (dims[0] contiguous).  u is None: x overwrites d.  Otherwise u += x."""
-    numel = 1
-    for v in dims:
-        numel *= int(v)
+    dc, nd, numel = _mesh(dims)
     _check_tensors((a, b, c, d, u), d, numel)
     L = load()
-    dc, nd = _dims(dims)
     if workspace is None:
         st = L.trid_solve_batch(_ptr(a), _ptr(b), _ptr(c), _ptr(d), _ptr(u), dc, nd, solve_dim,
                                 _dtype(d), _stream(stream))
@@ -154,12 +174,9 @@ def solve_noalloc(a, b, c, d, dims, solve_dim: int, u=None, stream=None):
     """As ``solve``, through trid_solve_batch_noalloc: for callers that must not
     let the library allocate device memory (the long-system scratch comes from
     a fixed 32 MiB device array; see include/trid.h)."""
-    numel = 1
-    for v in dims:
-        numel *= int(v)
+    dc, nd, numel = _mesh(dims)
     _check_tensors((a, b, c, d, u), d, numel)
     L = load()
-    dc, nd = _dims(dims)
     st = L.trid_solve_batch_noalloc(_ptr(a), _ptr(b), _ptr(c), _ptr(d), _ptr(u), dc, nd,
                                     solve_dim, _dtype(d), _stream(stream))
     if st != 0:
@@ -172,12 +189,9 @@ def adjoint(a, b, c, x, gx, dims, solve_dim: int, need_coef_grads: bool = True, 
     (g_a, g_b, g_c, g_d) (the first three None if ``need_coef_grads`` is
     False).  All arrays are CUDA tensors with the forward call's layout."""
     import torch
-    numel = 1
-    for v in dims:
-        numel *= int(v)
+    dc, nd, numel = _mesh(dims)
     _check_tensors((a, b, c, x, gx), x, numel)
     L = load()
-    dc, nd = _dims(dims)
     gd = torch.empty_like(x)
     ga = torch.empty_like(x) if need_coef_grads else None
     gb = torch.empty_like(x) if need_coef_grads else None
@@ -327,12 +341,9 @@ def adi_workspace_bytes(dims, dtype) -> int:
 
 def adi_step(u, dims, lam: float, nsteps: int, workspace, stream=None):
     """Advance u in place by ``nsteps`` ADI steps (Dirichlet-zero boundary)."""
-    numel = 1
-    for v in dims:
-        numel *= int(v)
+    dc, nd, numel = _mesh(dims)
     _check_tensors((u,), u, numel)
     L = load()
-    dc, nd = _dims(dims)
     st = L.adi_step(_ptr(u), dc, nd, float(lam), int(nsteps), _dtype(u), _ptr(workspace),
                     workspace.numel() * workspace.element_size(), _stream(stream))
     if st != 0:
@@ -345,12 +356,9 @@ def adi_step_batched(u, nbatch: int, dims, lam: float, nsteps: int, workspace=No
     """Advance each of the ``nbatch`` meshes stored back to back in ``u`` by
     ``nsteps`` ADI steps (see include/trid.h)."""
     import torch
-    per = 1
-    for v in dims:
-        per *= int(v)
+    dc, nd, per = _mesh(dims)
     _check_tensors((u,), u, per * int(nbatch))
     L = load()
-    dc, nd = _dims(dims)
     need = int(L.adi_batched_workspace_bytes(int(nbatch), dc, nd, _dtype(u)))
     if workspace is None and need:
         workspace = torch.empty(need, dtype=torch.uint8, device=u.device)
