@@ -114,6 +114,95 @@ k_lines(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ 
     }
 }
 
+// Contiguous systems whose rows are no whole 16-byte vectors (a length or an
+// array that is not a multiple of 16 bytes).  A warp's systems are one
+// contiguous run of at most 32 M elements of each array: it is brought to
+// shared memory by coalesced asynchronous copies of single elements, all in
+// flight at once, and each lane takes its tile from there (one element of
+// padding after every 8, so that tiles of 8 start in different banks); x goes
+// back the same way.  With scalar accesses of each lane's own rows (k_lines)
+// every one touches up to 32 sectors, eight times over.  FP32, that kernel ->
+// this one: 43571 systems of 201 rows 49.3 -> 37.0 us, accumulating 94.7 -> 41.7;
+// 90000 of 101 rows 40.7 -> 40.1 and 96.7 -> 44.6; 160000 of 17 rows 13.8 -> 16.4
+// and 38.0 -> 16.4; 250000 of 7 rows 13.9 -> 8.9 (FP64 is bound by its
+// arithmetic in both).  So it is taken when accumulating and for one, two or
+// 32 lanes per system; otherwise the lines of a warp meet in few enough
+// sectors.
+constexpr int LS_RUN = 32 * 8 + 32;   // elements of a warp's run with padding
+__device__ __forceinline__ int ls_pad(int q) { return q + (q >> 3); }
+template <typename T>
+__device__ __forceinline__ void ls_copy(T *dst, const T *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;"
+                 ::"r"(smem_u32(dst)), "l"(src), "n"(int(sizeof(T))) : "memory");
+}
+
+template <typename T, int M, int G>
+__global__ void __launch_bounds__(128)
+k_lines_staged(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ c,
+               const T *d, T *out, int accumulate, int64_t nsys, int64_t n) {
+    static_assert(M == 8, "padding and run length are those of 8-row tiles");
+    __shared__ T stage[4][4][LS_RUN];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t first = (int64_t(blockIdx.x) * 4 + w) * (32 / G);   // the warp's first system
+    const int g = lane % G, l = lane / G;
+    const int nn = int(n);
+    int64_t left = nsys - first;
+    if (left < 0) left = 0;
+    const int lines = left < 32 / G ? int(left) : 32 / G;
+    const int64_t base = first * n;
+    int cnt = lines * nn;
+    if (!TRID_BOUNDS(base + cnt <= nsys * n)) cnt = 0;
+    T *sa = stage[w][0], *sc = stage[w][1], *sd = stage[w][2], *sb = stage[w][3];
+    const T *pa = a + base + lane, *pc = c + base + lane, *pd = d + base + lane;
+    const T *pb = b ? b + base + lane : nullptr;
+    const int p0 = ls_pad(lane);
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+        if (lane + 32 * j < cnt) {
+            const int p = p0 + 36 * j;   // ls_pad(lane + 32 j)
+            ls_copy(sa + p, pa + 32 * j);
+            if (b) ls_copy(sb + p, pb + 32 * j);
+            ls_copy(sc + p, pc + 32 * j);
+            ls_copy(sd + p, pd + 32 * j);
+        }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    T ru[M];
+    if (accumulate) {
+#pragma unroll
+        for (int j = 0; j < M; ++j)
+            if (lane + 32 * j < cnt) ru[j] = out[base + lane + 32 * j];
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    T ra[M], rb[M], rc[M], rd[M];
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        const int i = g * M + j, q = l * nn + i, p = ls_pad(q);
+        const bool in = i < nn && q < cnt;
+        ra[j] = in && i > 0 ? sa[p] : T(0);
+        rb[j] = in && b ? sb[p] : T(1);
+        rc[j] = in && i < nn - 1 ? sc[p] : T(0);
+        rd[j] = in ? sd[p] : T(0);
+    }
+    T as, cs, ds, ae, ce, de, xs, xe;
+    tile_reduce<T, M>(ra, rb, rc, rd, as, cs, ds, ae, ce, de);
+    group_solve<T, G>(as, cs, ds, ae, ce, de, g, xs, xe);
+    tile_substitute<T, M>(ra, rc, rd, xs, xe);
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        const int i = g * M + j, q = l * nn + i;
+        if (i < nn && q < cnt) sd[ls_pad(q)] = rd[j];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        if (lane + 32 * j < cnt) {
+            const T x = sd[p0 + 36 * j];
+            out[base + lane + 32 * j] = accumulate ? ru[j] + x : x;
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Long systems, pass 1: reduced rows of every tile.  Thread = (system, tile);
 // STRIDED: systems are memory neighbours (lane = system) and the reduced
@@ -269,8 +358,12 @@ static void launch_lines(const T *a, const T *b, const T *c, const T *d, T *out,
                          const Lines &L, int vec_ok, cudaStream_t st) {
     const int64_t warps = (L.nsys + (32 / G) - 1) / (32 / G);
     const int64_t blocks = (warps + 7) / 8;
-    k_lines<T, TILE_M, G><<<dim3(unsigned(blocks)), 256, 0, st>>>(a, b, c, d, out, acc, L.nsys,
-                                                                   L.n, vec_ok);
+    if (vec_ok || !(acc || G <= 2 || G == 32))
+        k_lines<T, TILE_M, G><<<dim3(unsigned(blocks)), 256, 0, st>>>(a, b, c, d, out, acc,
+                                                                       L.nsys, L.n, vec_ok);
+    else
+        k_lines_staged<T, TILE_M, G><<<dim3(unsigned((warps + 3) / 4)), 128, 0, st>>>(
+            a, b, c, d, out, acc, L.nsys, L.n);
 }
 
 template <typename T, int NT>
