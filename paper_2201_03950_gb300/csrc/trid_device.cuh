@@ -104,6 +104,26 @@ __device__ __forceinline__ void tile_substitute(const T (&a)[M], const T (&c)[M]
     d[M - 1] = xe;
 }
 
+// The rows between a tile's known end unknowns (x_s, x_e): Thomas on rows 1 to
+// M - 2, 8 operations a row with the reciprocal's three, where reducing the
+// tile again and substituting takes 17.  b, a, c, d of the two end rows are not
+// used.
+template <typename T, int M>
+__device__ __forceinline__ void tile_interior(const T (&a)[M], const T (&b)[M], T (&c)[M],
+                                              T (&d)[M], T xs, T xe) {
+    d[0] = xs;
+    d[M - 1] = xe;
+    T cp = T(0);
+#pragma unroll
+    for (int i = 1; i < M - 1; ++i) {
+        const T r = rcp(b[i] - a[i] * cp);
+        cp = c[i] *= r;
+        d[i] = (d[i] - a[i] * d[i - 1]) * r;
+    }
+#pragma unroll
+    for (int i = M - 2; i >= 1; --i) d[i] = d[i] - c[i] * d[i + 1];
+}
+
 // ---- reduced solve across G consecutive lanes -------------------------------
 // Every lane of the warp must call this (full-warp shuffles).  `g` = the
 // lane's index inside its group of G lanes (tile index of the system).

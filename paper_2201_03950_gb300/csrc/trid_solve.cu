@@ -304,13 +304,11 @@ k_long_subst(const T *__restrict__ a, const T *__restrict__ b, const T *__restri
     const int64_t i0 = tile * M;
     T ra[M], rb[M], rc[M], rd[M];
     long_load<T, M>(a, b, c, d, L, base, i0, vec_ok, ra, rb, rc, rd);
-    T as, cs, ds, ae, ce, de;
-    tile_reduce<T, M>(ra, rb, rc, rd, as, cs, ds, ae, ce, de);
     const int64_t R = 2 * ntiles;
     int64_t ps, pe;
     if (STRIDED) { ps = (2 * tile) * L.nsys + sys; pe = ps + L.nsys; }
     else { ps = sys * R + 2 * tile; pe = ps + 1; }
-    tile_substitute<T, M>(ra, rc, rd, rx[ps], rx[pe]);
+    tile_interior<T, M>(ra, rb, rc, rd, rx[ps], rx[pe]);
     if (vec_ok && L.stride == 1 && i0 + M <= L.n) {
         if (accumulate) {
             T ru[M];
