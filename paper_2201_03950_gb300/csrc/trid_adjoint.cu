@@ -254,6 +254,20 @@ static void launch_adj_lines(const T *a, const T *b, const T *c, const T *x, con
 template <typename T, int NT>
 static void launch_adj_strided(const T *a, const T *b, const T *c, const T *x, const T *gx, T *ga,
                                T *gb, T *gc, T *gd, const Lines &L, cudaStream_t st) {
+    // 16 systems per block, or 32 when one system spans much memory: every block
+    // then touches all pages of the nine arrays, and rows of 128 bytes instead
+    // of 64 halve the touches.  FP32: 512 x 512 x 64 along z (64 MiB a system)
+    // 172 -> 94 us, 256^3 along z (64 MiB) 136 -> 116, but 256 x 256 x 128 along z
+    // (32 MiB) 53.1 against 53.6 and 256^3 along y (256 KiB) 100 against 112.
+    // Bringing the arrays by TMA boxes as the solves do took 118 and 139 us
+    // along z and 112 along y: five boxes leave room for one stage per block.
+    if constexpr (sizeof(T) == 4) {
+        if (L.n * L.stride * int64_t(sizeof(T)) >= (int64_t(48) << 20)) {
+            k_adjoint_strided<T, ADJ_M, NT, 32><<<strided_grid(L, 32), NT * 32, 0, st>>>(
+                a, b, c, x, gx, ga, gb, gc, gd, L, L.nsys / L.inner);
+            return;
+        }
+    }
     constexpr int SG = (NT * SysCfg<T>::SG < 32) ? 32 / NT : SysCfg<T>::SG;
     k_adjoint_strided<T, ADJ_M, NT, SG><<<strided_grid(L, SG), NT * SG, 0, st>>>(
         a, b, c, x, gx, ga, gb, gc, gd, L, L.nsys / L.inner);
