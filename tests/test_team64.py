@@ -1,0 +1,72 @@
+"""FP64 systems of 257 to 4096 rows in one pass (k_team64), against the FP64
+oracle: row counts around every number of tiles per warp and every number of
+systems per block, contiguous in whole vectors and not, strided, system counts
+that fill no block, weakly coupled and nearly singular systems, and the limits
+beyond which the passes through scratch run.  GPU only."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2201_03950_gb300 import inputs, trid
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def solve(dims, k, acc=False, offset=0, margin=None):
+    n = int(np.prod(dims))
+    a, b, c, d = inputs.dominant_system((n,), seed=n + k, dtype=np.float64)
+    if margin is not None:
+        b = np.abs(a) + np.abs(c) + margin
+    idx = np.moveaxis(np.arange(n).reshape(dims[::-1]), len(dims) - 1 - k, 0)
+    ref = oracle.solve_mesh(a, b, c, d, dims, k)
+    a[idx[0].reshape(-1)] = np.nan     # not part of the system, so never used
+    c[idx[-1].reshape(-1)] = np.nan
+
+    def dev(v):
+        t = torch.empty(n + offset, dtype=torch.float64, device="cuda")[offset:]
+        return t.copy_(torch.from_numpy(v))
+
+    ta, tb, tc, td = (dev(v) for v in (a, b, c, d))
+    u0 = inputs.random_rhs((n,), seed=5, dtype=np.float64) if acc else np.zeros(n)
+    tu = dev(u0) if acc else None
+    out = trid.solve(ta, tb, tc, td, dims, k, u=tu)
+    if acc:
+        assert np.array_equal(td.cpu().numpy(), d)
+    return out.cpu().numpy() - u0, ref
+
+
+def check(got, ref, tol=1e-12):
+    assert np.all(np.isfinite(got))
+    assert np.max(np.abs(got - ref)) <= tol * np.max(np.abs(ref))
+
+
+ROWS = [257, 260, 271, 272, 273, 300, 511, 512, 513, 700, 1001, 1024, 1536, 2047, 3072, 3073, 4095,
+        4096, 4097]
+
+
+@pytest.mark.parametrize("n", ROWS)
+@pytest.mark.parametrize("acc", [False, True], ids=["store", "acc"])
+def test_rows(n, acc):
+    check(*solve((n, 7), 0, acc))
+    check(*solve((7, n), 1, acc))
+
+
+@pytest.mark.parametrize("n", [300, 400, 512, 700, 1000])
+def test_many_systems(n):
+    check(*solve((n, 2503), 0))          # several systems per block, the last block not full
+    check(*solve((2503, n), 1))
+    check(*solve((13, n, 197), 1))       # neighbours across the rows of a plane
+
+
+def test_unaligned_arrays():
+    check(*solve((512, 40), 0, offset=1))
+    check(*solve((40, 512), 1, offset=1))
+
+
+@pytest.mark.parametrize("margin,tol", [(1e-3, 1e-10), (1e-6, 1e-7)])
+def test_weak_dominance(margin, tol):
+    """Couplings that stay above the stopping bound for every round; the
+    condition number (at most 3 / margin) times 2^-53, a few hundred times over."""
+    check(*solve((1500, 9), 0, margin=margin), tol=tol)
+    check(*solve((9, 1500), 1, margin=margin), tol=tol)
