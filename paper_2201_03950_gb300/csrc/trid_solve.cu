@@ -593,6 +593,68 @@ static bool launch_twist(const T *a, const T *b, const T *c, const T *d, T *out,
     }
 }
 
+// Strided FP32 systems of 256 < n <= 1024 rows with 16, 24 or 32 rows per
+// thread through k_strided: one block per 8 or 16 systems, no cluster and no
+// exchange between blocks, for as many systems as its blocks take in one or
+// two rounds; beyond that the clusters, which stream their strips, are faster
+// (with inputs that were not in the L2; this kernel against k_chunk_cluster):
+//   512 rows   1024 systems 3.7 against 5.7 us, 4096 10.5 / 12.3, 8192 23.2 / 19.5
+//   768 rows   1024 systems 4.7 / 6.7, 4864 17.9 / 19.5, 8192 31.8 / 28.0
+//   1024 rows  256 systems 5.6 / 5.5, 1024 5.6 / 7.2, 2048 10.1 / 12.8, 4096 23.0 / 20.0
+// Accumulating, the clusters store without TMA and lose more:
+//   512 rows   16384 systems 41 / 63;  768 rows  4864 systems 31 / 35
+//   1024 rows  1024 systems 5.3 / 9.4, 2048 25.1 / 20.5 (16 systems a block spill)
+// Arrays that the clusters do not take went through scratch in passes
+// (1001 x 1001: 10.9 -> 7.3 us).
+template <int M, int SG>
+static bool launch_strided_tall_form(const float *a, const float *b, const float *c,
+                                     const float *d, float *out, int acc, const Lines &L,
+                                     cudaStream_t st) {
+    ArrayCoef<float> coef{a, b, c};
+    if (acc)
+        k_strided<float, M, 32, SG, true, ArrayCoef<float>>
+            <<<strided_grid(L, SG), 32 * SG, 0, st>>>(coef, d, out, L, L.nsys / L.inner);
+    else
+        k_strided<float, M, 32, SG, false, ArrayCoef<float>>
+            <<<strided_grid(L, SG), 32 * SG, 0, st>>>(coef, d, out, L, L.nsys / L.inner);
+    return launch_ok();
+}
+
+template <typename T>
+static bool launch_strided_tall(const T *a, const T *b, const T *c, const T *d, T *out, int acc,
+                                const Lines &L, bool has_scratch, cudaStream_t st) {
+    if constexpr (!std::is_same<T, float>::value) {
+        return false;
+    } else {
+        const DeviceInfo *di = device_info();
+        if (!di || L.stride == 1 || !b || L.n <= MAX_SINGLE_PASS || L.n > 1024 ||
+            !strided_offsets_fit(L))
+            return false;
+        const bool tma = is_aligned16(a) && is_aligned16(b) && is_aligned16(c) &&
+                         is_aligned16(d) && is_aligned16(out) && (L.inner * 4) % 16 == 0;
+        // (arrays that the clusters cannot take had to bring scratch)
+        if (!tma && !has_scratch) return false;
+        const int64_t outer = L.nsys / L.inner;
+        const int64_t b8 = (L.inner + 7) / 8 * outer, b16 = (L.inner + 15) / 16 * outer;
+        const int64_t sms = di->sm_count;
+        const bool few = b8 <= sms;
+        if (L.n > 768 && acc && !few) return false;
+        if (tma) {
+            if (L.n <= 512 ? !acc && b16 > 2 * sms : L.n <= 768 ? b16 > 2 * sms : b16 > sms)
+                return false;
+            if (L.n > 768 && !acc && b8 < 64) return false;
+        }
+        if (L.n <= 512)
+            return few ? launch_strided_tall_form<16, 8>(a, b, c, d, out, acc, L, st)
+                       : launch_strided_tall_form<16, 16>(a, b, c, d, out, acc, L, st);
+        if (L.n <= 768)
+            return few ? launch_strided_tall_form<24, 8>(a, b, c, d, out, acc, L, st)
+                       : launch_strided_tall_form<24, 16>(a, b, c, d, out, acc, L, st);
+        return few ? launch_strided_tall_form<32, 8>(a, b, c, d, out, acc, L, st)
+                   : launch_strided_tall_form<32, 16>(a, b, c, d, out, acc, L, st);
+    }
+}
+
 // FP64 systems of 256 < n <= 4096 rows (strided: 3072) through k_team64.
 // Systems per block: the number that leaves the fewest of the block's threads
 // without a tile, blocks of up to 256 threads first (several share an SM and
@@ -687,6 +749,9 @@ static trid_status solve_lines(const T *a, const T *b, const T *c, const T *d, T
     }
     // up to 4096 contiguous FP32 rows: one pass, systems staged by bulk copies
     if (launch_lines_tma<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
+    if (launch_strided_tall<T>(a, b, c, d, out, acc, L, ws_bytes >= long_ws_bytes<T>(L.nsys, L.n),
+                               st))
+        return TRID_OK;
     // strided FP32 up to 4096 rows: one cluster per strip of systems
     if (launch_chunk_cluster<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
     // long systems: tiled Thomas-PCR in passes
