@@ -600,12 +600,14 @@ static bool launch_twist(const T *a, const T *b, const T *c, const T *d, T *out,
 // (with inputs that were not in the L2; this kernel against k_chunk_cluster):
 //   512 rows   1024 systems 3.7 against 5.7 us, 4096 10.5 / 12.3, 8192 23.2 / 19.5
 //   768 rows   1024 systems 4.7 / 6.7, 4864 17.9 / 19.5, 8192 31.8 / 28.0
-//   1024 rows  256 systems 5.6 / 5.5, 1024 5.6 / 7.2, 2048 10.1 / 12.8, 4096 23.0 / 20.0
-// Accumulating, the clusters store without TMA and lose more:
-//   512 rows   16384 systems 41 / 63;  768 rows  4864 systems 31 / 35
+//   1024 rows  256 systems 5.6 / 5.5, 1024 5.6 / 7.2, 4096 23.0 / 20.0
+// and accumulating, where the clusters store without TMA,
+//   512 rows   4096 systems 11.7 / 20.8;  768 rows  4864 systems 31.0 / 35.4
 //   1024 rows  1024 systems 5.3 / 9.4, 2048 25.1 / 20.5 (16 systems a block spill)
-// Arrays that the clusters do not take went through scratch in passes
-// (1001 x 1001: 10.9 -> 7.3 us).
+// The choice is the same for storing and accumulating and whatever `out` is: a
+// differentiable ADI recomputes with stored solves the states that its forward
+// accumulated, and must get the same bits.  Arrays that the clusters do not
+// take went through scratch in passes (1001 x 1001: 10.9 -> 7.3 us).
 template <int M, int SG>
 static bool launch_strided_tall_form(const float *a, const float *b, const float *c,
                                      const float *d, float *out, int acc, const Lines &L,
@@ -630,28 +632,22 @@ static bool launch_strided_tall(const T *a, const T *b, const T *c, const T *d, 
         if (!di || L.stride == 1 || !b || L.n <= MAX_SINGLE_PASS || L.n > 1024 ||
             !strided_offsets_fit(L))
             return false;
-        const bool tma = is_aligned16(a) && is_aligned16(b) && is_aligned16(c) &&
-                         is_aligned16(d) && is_aligned16(out) && (L.inner * 4) % 16 == 0;
+        const bool clusters = is_aligned16(a) && is_aligned16(b) && is_aligned16(c) &&
+                              is_aligned16(d) && (L.inner * 4) % 16 == 0;
         // (arrays that the clusters cannot take had to bring scratch)
-        if (!tma && !has_scratch) return false;
-        const int64_t outer = L.nsys / L.inner;
+        if (!clusters && !has_scratch) return false;
+        const int64_t outer = L.nsys / L.inner, sms = di->sm_count;
         const int64_t b8 = (L.inner + 7) / 8 * outer, b16 = (L.inner + 15) / 16 * outer;
-        const int64_t sms = di->sm_count;
         const bool few = b8 <= sms;
-        if (L.n > 768 && acc && !few) return false;
-        if (tma) {
-            if (L.n <= 512 ? !acc && b16 > 2 * sms : L.n <= 768 ? b16 > 2 * sms : b16 > sms)
-                return false;
-            if (L.n > 768 && !acc && b8 < 64) return false;
-        }
+        if (L.n > 768 && !few) return false;
+        if (clusters && (b16 > 2 * sms || (L.n > 768 && b8 < 64))) return false;
         if (L.n <= 512)
             return few ? launch_strided_tall_form<16, 8>(a, b, c, d, out, acc, L, st)
                        : launch_strided_tall_form<16, 16>(a, b, c, d, out, acc, L, st);
         if (L.n <= 768)
             return few ? launch_strided_tall_form<24, 8>(a, b, c, d, out, acc, L, st)
                        : launch_strided_tall_form<24, 16>(a, b, c, d, out, acc, L, st);
-        return few ? launch_strided_tall_form<32, 8>(a, b, c, d, out, acc, L, st)
-                   : launch_strided_tall_form<32, 16>(a, b, c, d, out, acc, L, st);
+        return launch_strided_tall_form<32, 8>(a, b, c, d, out, acc, L, st);
     }
 }
 
