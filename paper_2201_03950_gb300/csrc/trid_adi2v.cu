@@ -286,6 +286,7 @@ __global__ void k_v2_rhs_keep(const T *up, const T *dp, T *u, const T *ax, const
 // p + 1 (if interior) + (b_x - c_x) at p (if interior), face (p, p + 1);
 // F_y alike for face (p, p + nx).
 //
+// (The face sums of lines of a multiple of 4 points: k_v2_rhs_adj4 below.)
 // Each thread walks V2_ROWS consecutive rows of one column, keeping the
 // column's values of the rows above and below in registers (the x
 // neighbours are read directly and mostly hit L1).
@@ -380,6 +381,121 @@ k_v2_rhs_adj(const T *g, const T *gd, const T *gw, const T *u, const T *w, const
         ay_c = ay_p; ay_p = col(ay, j + 2);
         cy_m = cy_c; cy_c = col(cy, j + 1);
     }
+    }
+}
+
+// The face-sum form for lines of a multiple of 4 points: four neighbouring
+// columns of one row per thread, a block of 32 x 4 threads, so that a row takes
+// 16-byte loads where each column took a dozen of 4 bytes, and the terms that
+// two x faces share are formed once.  15 words per point and step from the L2;
+// the loads in flight bound it.  1024^2 FP32 19.2 -> 11.3 us; walking down two or
+// four rows, with the rows above and below kept, 13.2 and 12.9 (fewer threads),
+// one row in blocks of 128 x 1 13.1 (no neighbouring rows in the L1).
+constexpr int V2F_X = 32, V2F_Y = 4;
+
+template <typename T>
+__global__ void __launch_bounds__(V2F_X *V2F_Y, sizeof(T) == 4 ? 4 : 2)
+k_v2_rhs_adj4(const T *g, const T *gd, const T *gw, const T *u, const T *w, const T *dl,
+              const T *ax, const T *cx, const T *ay, const T *cy, T *G, T *gn, int nx, int ny,
+              size_t n) {
+    pdl_wait();
+    const int i0 = 4 * int(blockIdx.x * V2F_X + threadIdx.x);
+    if (i0 >= nx) return;
+    for (int j = int(blockIdx.y * V2F_Y + threadIdx.y); j < ny; j += int(gridDim.y) * V2F_Y) {
+        const size_t p = size_t(j) * nx + i0;
+        auto row = [&](const T *a, int dj, T (&v)[4]) {   // row j + dj; 0 outside the mesh
+            if (j + dj >= 0 && j + dj < ny) {
+                load_contig_vec<T, 4>(a + (p + ptrdiff_t(dj) * nx), v);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = T(0);
+            }
+        };
+        auto in_x = [&](int e) { return i0 + e > 0 && i0 + e < nx - 1; };
+        const bool jin = j > 0 && j < ny - 1;
+        const bool jpin = j + 1 > 0 && j + 1 < ny - 1, jmin = j - 1 > 0 && j - 1 < ny - 1;
+        const bool left = i0 > 0, right = i0 + 4 < nx;
+        T gv[4], r_c[4], r_m[4], r_p[4], axv[4], cxv[4], ay_c[4], ay_p[4], cy_c[4], cy_m[4];
+        row(g, 0, gv);
+        row(gd, 0, r_c);
+        row(gd, -1, r_m);
+        row(gd, 1, r_p);
+        row(ax, 0, axv);
+        row(cx, 0, cxv);
+        row(ay, 0, ay_c);
+        row(ay, 1, ay_p);
+        row(cy, 0, cy_c);
+        row(cy, -1, cy_m);
+        T uv[4], u_p[4], wv[4], d_c[4], d_p[4], gw_c[4], gw_p[4], Gx[4], Gy[4];
+        row(u, 0, uv);
+        row(u, 1, u_p);
+        row(w, 0, wv);
+        row(dl, 0, d_c);
+        row(dl, 1, d_p);
+        row(gw, 0, gw_c);
+        row(gw, 1, gw_p);
+        row(G, 0, Gx);
+        row(G + n, 0, Gy);
+        const T cx_l = left ? cx[p - 1] : T(0), ax_r = right ? ax[p + 4] : T(0);
+        const T gd_l = left ? gd[p - 1] : T(0), gd_r = right ? gd[p + 4] : T(0);
+        const T w_l = left ? w[p - 1] : T(0), w_r = right ? w[p + 4] : T(0);
+        const T u_l = left ? u[p - 1] : T(0), u_r = right ? u[p + 4] : T(0);
+        // g_d on the interior, elements -1 .. 4
+        T gi[6];
+        gi[0] = (jin && in_x(-1)) ? gd_l : T(0);
+        gi[5] = (jin && right && in_x(4)) ? gd_r : T(0);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) gi[e + 1] = (jin && in_x(e)) ? r_c[e] : T(0);
+        // the step's gradients of a_x and b_x at elements 0 .. 4 (x solve and stencil)
+        T sa[5], sb[5], out[4];
+#pragma unroll
+        for (int e = 0; e < 5; ++e) {
+            const T r = e < 4 ? r_c[e < 4 ? e : 0] : gd_r;
+            const T wm = e > 0 ? wv[e > 0 ? e - 1 : 0] : w_l, w0 = e < 4 ? wv[e < 4 ? e : 0] : w_r;
+            const T um = e > 0 ? uv[e > 0 ? e - 1 : 0] : u_l, u0 = e < 4 ? uv[e < 4 ? e : 0] : u_r;
+            sa[e] = i0 + e > 0 ? -r * wm : T(0);
+            sb[e] = -r * w0;
+            if (gi[e + 1] != T(0)) sa[e] += gi[e + 1] * (u0 - um);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i = i0 + e;
+            const T wp = e < 3 ? wv[e < 3 ? e + 1 : 3] : w_r;
+            const T ur = e < 3 ? uv[e < 3 ? e + 1 : 3] : u_r;
+            T sc = i < nx - 1 ? -r_c[e] * wp : T(0);
+            if (gi[e + 1] != T(0)) sc += gi[e + 1] * (uv[e] - ur);
+            // the stencil's reverse
+            const T cl = e > 0 ? cxv[e > 0 ? e - 1 : 0] : cx_l;
+            const T ar = e < 3 ? axv[e < 3 ? e + 1 : 3] : ax_r;
+            const T gyp = jpin && in_x(e) ? r_p[e] : T(0);
+            T acc = gv[e] + (axv[e] + cxv[e] + ay_c[e] + cy_c[e]) * gi[e + 1];
+            if (i > 0) acc -= cl * gi[e];
+            if (i < nx - 1) acc -= ar * gi[e + 2];
+            if (j > 0) acc -= cy_m[e] * (jmin && in_x(e) ? r_m[e] : T(0));
+            if (j < ny - 1) acc -= ay_p[e] * gyp;
+            out[e] = acc;
+            if (i < nx - 1) {   // face (p, p + 1): (b - c) at p, (b - a) at p + 1
+                T f = i > 0 ? sb[e] - sc : T(0);
+                if (i + 1 < nx - 1) f += sb[e + 1] - sa[e + 1];
+                Gx[e] += f;
+            }
+            if (j < ny - 1) {   // face (p, p + nx)
+                const T tb = -gw_c[e] * d_c[e];
+                T tc = -gw_c[e] * d_p[e];
+                if (gi[e + 1] != T(0)) tc += gi[e + 1] * (uv[e] - u_p[e]);
+                T f = j > 0 ? tb - tc : T(0);
+                if (j + 1 < ny - 1) {
+                    T a1 = -gw_p[e] * d_c[e];
+                    const T b1 = -gw_p[e] * d_p[e];
+                    if (gyp != T(0)) a1 += gyp * (u_p[e] - uv[e]);
+                    f += b1 - a1;
+                }
+                Gy[e] += f;
+            }
+        }
+        store_contig_vec<T, 4>(gn + p, out);
+        store_contig_vec<T, 4>(G + p, Gx);
+        store_contig_vec<T, 4>(G + n + p, Gy);
     }
 }
 
@@ -614,6 +730,11 @@ static trid_status v2_backward(const T *guT, T *gu0, T *gk, T *gcoef, const T *k
     // the column-walking reverse kernel: V2_ROWS rows per thread
     const int64_t bands = (int64_t(ny) + V2_ROWS - 1) / V2_ROWS;
     const dim3 ga(unsigned((nx + 255) / 256), unsigned(bands < 65535 ? bands : 65535));
+    // (every array is in the workspace, so rows are whole 16-byte vectors)
+    const bool four = !gcoef && nx % 4 == 0;
+    const int64_t rows4 = (int64_t(ny) + V2F_Y - 1) / V2F_Y;
+    const dim3 b4(V2F_X, V2F_Y);
+    const dim3 g4(unsigned((nx / 4 + V2F_X - 1) / V2F_X), unsigned(rows4 < 65535 ? rows4 : 65535));
     k_v2_coef<T><<<g2, b2, 0, st>>>(kap, co[0], co[1], co[2], co[3], co[4], co[5], nx, ny, lam);
     k_v2_transpose<T><<<g2, b2, 0, st>>>(co[0], co[2], co[3], co[5], tr, tr + ms, tr + 2 * ms,
                                          tr + 3 * ms, nx, ny);
@@ -683,8 +804,9 @@ static trid_status v2_backward(const T *guT, T *gu0, T *gk, T *gcoef, const T *k
             if (s != TRID_OK) return s;
             s = solve_into_ws(tr, co[1], tr + ms, gw, gd, dims, 2, 0, dt, scr, l.scratch, st);
             if (s != TRID_OK) return s;
-            auto kern = gcoef ? k_v2_rhs_adj<T, true> : k_v2_rhs_adj<T, false>;
-            if (!launch_pdl(kern, ga, b2, st, g, gd, gw, U + size_t(q) * ms, W + size_t(q) * ms,
+            auto kern = gcoef ? k_v2_rhs_adj<T, true>
+                              : four ? k_v2_rhs_adj4<T> : k_v2_rhs_adj<T, false>;
+            if (!launch_pdl(kern, four ? g4 : ga, four ? b4 : b2, st, g, gd, gw, U + size_t(q) * ms, W + size_t(q) * ms,
                             D + size_t(q) * ms, co[0], co[2], co[3], co[5], G, gn, nx, ny, ms))
                 return TRID_ERR_CUDA;
             T *tmp = g;

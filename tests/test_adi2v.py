@@ -177,3 +177,17 @@ def test_invalid_arguments():
     small = torch.empty(16, dtype=torch.uint8, device="cuda")
     with pytest.raises(trid.TridError):
         trid.adi2v_forward(t, t, dims, 0.1, 3, 2, workspace=small)
+
+
+# The reverse stencil kernel of the face sums takes four columns per thread when
+# a line is a multiple of 4 points: its smallest widths, widths that fill no
+# block, few rows, and (33 x 20 and others above) the widths it does not take.
+@pytest.mark.parametrize("dtype", [np.float32, np.float64], ids=["f32", "f64"])
+@pytest.mark.parametrize("dims", [(4, 3), (4, 4), (8, 5), (12, 30), (124, 7), (128, 9), (132, 66),
+                                  (260, 33)], ids=lambda d: f"{d[0]}x{d[1]}")
+def test_face_sums_of_whole_vectors(dims, dtype):
+    u0, kap, tg = problem(dims, sum(dims), dtype)
+    loss, rgu, rgk, _ = oracle.adi2v_grad(u0, kap, tg, dims, 0.3, 5)
+    _, gu, gk, _ = gpu_run(u0, kap, tg, dims, 0.3, 5, 2, dtype)
+    assert normwise(gu, rgu) <= TOL_GRAD[dtype]
+    assert normwise(gk, rgk) <= TOL_GRAD[dtype]
