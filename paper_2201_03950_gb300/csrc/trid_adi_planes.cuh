@@ -14,12 +14,13 @@
 // z are independent (each keeps its own boundary planes).
 //
 // What bounds pass A is the number of instructions and the shared-memory
-// accesses of its three phases (48^3 x 72: 36 us, half of the issue slots and
-// 57% of the shared-memory pipe); loading the planes a few rows at a time
-// instead of all at once took 56 us (latency of the loads), and computing
-// every copy's address anew 43.  Measured per step, FP32: 72 meshes of 48^3
-// 108.8 -> 40.4 us, 24 of 64^3 at lambda 0.3 65.9 -> 32.9, one of 100^3 23.6 ->
-// 13.5; FP64 72 of 48^3 805 -> 251, one of 100^3 203 -> 82.
+// accesses of its three phases (48^3 x 72: 30 us, 46% of the issue slots and 45%
+// of the shared-memory pipe busy, 21 warps per SM); loading the planes a few rows
+// at a time instead of all at once took 56 us (latency of the loads), computing
+// every copy's address anew 43, and handling the boundary columns' lanes apart
+// from the others 34 (every warp has one).  Measured per step, FP32: 72 meshes of
+// 48^3 108.8 -> 35.1 us, 24 of 64^3 at lambda 0.3 65.9 -> 31.4, one of 100^3 23.5
+// -> 12.8; FP64 72 of 48^3 805 -> 251, one of 100^3 203 -> 82.
 #pragma once
 #include "trid_adi_plane.cuh"
 #include "trid_tma.cuh"
@@ -68,51 +69,53 @@ k_adi_planes(const T *u, T *w, int nx, int ny, int nz,
     const int z = 1 + int(blockIdx.x) - mesh * (nz - 2);
     const int plane = nx * ny;
     const size_t base = (size_t(mesh) * nz + z) * size_t(plane);
-    // the group of four that the line begins in is read whole: what lies
-    // before the boundary node is 0 (its factors are 0 too)
-    for (int r = tid; r < ny; r += blockDim.x)
-        for (int q = offx & ~3; q < offx; ++q) {
-            sm[urow(r) + q] = sm[urow(r) + HX + q] = T(0);
-            if (r > 0 && r < ny - 1) {
-                sm[drow(r) + q] = sm[drow(r) + HX + q] = T(0);
-                sm[eoff + drow(r) + q] = sm[eoff + drow(r) + HX + q] = T(0);
-            }
+    // The group of four that the line begins in is read whole: what lies before
+    // the boundary node is 0 (its factors are 0 too).  The boundary columns' z
+    // neighbours and the plane's corners enter no explicit part: 0 as well.
+    for (int r = tid; r < ny; r += blockDim.x) {
+        const bool inner = r > 0 && r < ny - 1;
+        T *du = sm + urow(r), *dd = sm + drow(r);
+        for (int q = offx & ~3; q <= offx; ++q) {
+            if (q < offx || !inner) du[q] = du[HX + q] = T(0);
+            if (inner) dd[q] = dd[HX + q] = dd[eoff + q] = dd[eoff + HX + q] = T(0);
         }
+    }
     pdl_trigger();
     pdl_wait();   // u is written by the previous kernel on the stream
     const T *up = u + base;
     char *wp = reinterpret_cast<char *>(w + base);
-    // all three planes by asynchronous copies, every one in flight at once:
-    // columns by lane, the rows of each half by warp (constant address steps)
-    for (int x = lane; x < nx; x += 32) {
-        const bool bx = x == 0 || x == nx - 1;
-        const int px = pos(x);
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            const int rows = hh ? ny - hy : hy, gs = (hh ? -nx : nx) * nwarp;
+    // all three planes by asynchronous copies, every one in flight at once,
+    // rows by warp (constant address steps): 32 columns of one half's rows at a
+    // time, or where that leaves 16 lanes or more without a column, 16 columns
+    // of both halves' rows
+    auto fetch = [&](int hh, int x0, int dx) {
+        const int rows = hh ? ny - hy : hy, gs = (hh ? -nx : nx) * nwarp;
+        for (int x = x0; x < nx; x += dx) {
+            const bool inner = x > 0 && x < nx - 1;
+            const int px = pos(x);
             const T *q = up + (hh ? (ny - 1 - warp) * nx : warp * nx) + x;
             T *du = sm + (hh ? l.u1 : 0) + px + warp * p;
             T *dd = sm + (hh ? l.d1 : l.d0) + px + (warp - 1) * p;
             int k = warp;
-            if (k == 0) {   // the boundary row: its corners enter no explicit part
-                if (bx) *du = T(0);
-                else cp_async_elem(du, q);
+            if (k == 0) {   // the boundary row
+                if (inner) cp_async_elem(du, q);
                 k += nwarp; q += gs; du += nwarp * p; dd += nwarp * p;
             }
-            if (bx) {       // nor do a boundary column's z neighbours
-                for (; k < rows; k += nwarp, q += gs, du += nwarp * p, dd += nwarp * p) {
-                    cp_async_elem(du, q);
-                    dd[0] = dd[eoff] = T(0);
-                }
-            } else {
 #pragma unroll 4
-                for (; k < rows; k += nwarp, q += gs, du += nwarp * p, dd += nwarp * p) {
-                    cp_async_elem(du, q);
+            for (; k < rows; k += nwarp, q += gs, du += nwarp * p, dd += nwarp * p) {
+                cp_async_elem(du, q);
+                if (inner) {
                     cp_async_elem(dd, q - plane);
                     cp_async_elem(dd + eoff, q + plane);
                 }
             }
         }
+    };
+    if ((nx + 31) / 32 * 32 - nx < 16) {
+        fetch(0, lane, 32);
+        fetch(1, lane, 32);
+    } else {
+        fetch(half, lane & 15, 16);
     }
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();
