@@ -22,8 +22,8 @@
 //                        two rows per thread, solved there by block-wide PCR
 //                        (stopping once the couplings are below 1/16 ulp) and
 //                        substituted back level by level; pass 2 re-reads the
-//                        system (L2-resident), repeats the tile pass and
-//                        writes x.
+//                        system (L2-resident) and runs Thomas between each
+//                        tile's known ends.
 //     M2  (<= 4088)      one system per block, one pass: every thread keeps
 //                        its tile in registers through the reduced solve.
 //     M1  (<= 1016)      one system per team of 4 warps (4 teams per block,
@@ -587,13 +587,12 @@ k_varlen_solve(const T *__restrict__ a, const T *__restrict__ b, const T *__rest
         __syncthreads();
         if (ok) block_reduced_solve<T, VL_M>(sbase, rmax0, l0.R, nlevels);
         if (tid == helper) s_it[cur ^ 1] = VItem{(long long)nx_item, nx_meta.x, nx_meta.y};
-        // pass 2: recompute every tile and substitute its end values
+        // pass 2: the rows between every tile's known ends (8 FP64 operations a row
+        // where reducing the tile again took 17: 8192 systems in FP64 1125 -> 1031 us)
         for (int64_t t = tid; t < ntiles; t += blockDim.x) {
             T ra[VL_M], rb[VL_M], rc[VL_M], rd[VL_M];
             load_sys_tile<T, VL_M>(a, b, c, d, s0, n, pad, total, t, ra, rb, rc, rd);
-            T as, cs, ds, ae, ce, de;
-            tile_reduce<T, VL_M>(ra, rb, rc, rd, as, cs, ds, ae, ce, de);
-            tile_substitute<T, VL_M>(ra, rc, rd, l0.D(2 * t), l0.D(2 * t + 1));
+            tile_interior<T, VL_M>(ra, rb, rc, rd, l0.D(2 * t), l0.D(2 * t + 1));
             store_sys_tile<T, VL_M>(out, accumulate, s0, n, pad, total, t, rd);
         }
         __syncthreads();  // level 0 is rewritten by the next system
