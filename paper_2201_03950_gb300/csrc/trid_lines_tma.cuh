@@ -1,4 +1,4 @@
-// trid_lines_tma.cuh -- contiguous systems of 256 < N <= 4096 rows (FP32) in
+// trid_lines_tma.cuh -- contiguous systems of 512 < N <= 4096 rows (FP32) in
 // one pass (arXiv 2201.03950, Section 3.1, tiled Thomas-PCR).
 //
 // A persistent block (one per SM) of 16 consumer warps and one producer warp.

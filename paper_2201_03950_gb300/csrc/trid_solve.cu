@@ -20,7 +20,8 @@
 //             systems (2 rows per tile) are solved by a recursive call, and
 //             k_long_subst recomputes each tile and substitutes the tile-end
 //             unknowns back.
-//  k_lines_tma  contiguous FP32 systems of 256 < N <= 4096 in one pass:
+//             N <= 512 with 16 rows per lane (contiguous FP32).
+//  k_lines_tma  contiguous FP32 systems of 512 < N <= 4096 in one pass:
 //             whole systems staged in shared memory by bulk copies, one team
 //             of warps per system (trid_lines_tma.cuh).
 //  k_team64   FP64 systems of 256 < N <= 4096 in one pass, a block per few
@@ -131,7 +132,6 @@ k_lines(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ 
 // arithmetic in both).  So it is taken when accumulating and for one, two or
 // 32 lanes per system; otherwise the lines of a warp meet in few enough
 // sectors.
-constexpr int LS_RUN = 32 * 8 + 32;   // elements of a warp's run with padding
 __device__ __forceinline__ int ls_pad(int q) { return q + (q >> 3); }
 template <typename T>
 __device__ __forceinline__ void ls_copy(T *dst, const T *src) {
@@ -143,8 +143,8 @@ template <typename T, int M, int G>
 __global__ void __launch_bounds__(128)
 k_lines_staged(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ c,
                const T *d, T *out, int accumulate, int64_t nsys, int64_t n) {
-    static_assert(M == 8, "padding and run length are those of 8-row tiles");
-    __shared__ T stage[4][4][LS_RUN];
+    constexpr int RUN = 32 * M + 4 * M;   // elements of a warp's run with padding
+    __shared__ T stage[4][4][RUN];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t first = (int64_t(blockIdx.x) * 4 + w) * (32 / G);   // the warp's first system
     const int g = lane % G, l = lane / G;
@@ -354,6 +354,36 @@ static size_t long_ws_bytes(int64_t nsys, int64_t n) {
     return 3 * one + long_ws_bytes<T>(nsys, R);
 }
 
+// Contiguous FP32 systems of 256 < n <= 512 rows: one warp each with 16 rows per
+// lane.  Teams of two warps fed by bulk copies, which took them before, pay a
+// named barrier and a reduced solve in shared memory per system; that -> this:
+// 8192 systems of 300 rows 17.7 -> 11.6 us, of 512 rows 18.3 -> 14.5, 30000 of 512
+// rows 50.7 -> 44.9 (accumulating 70.5 -> 53.7), 1024 of 512 rows 4.1 -> 3.1.
+// Systems that are no whole 16-byte vectors went through scratch in passes (and
+// are taken only where those could run, so that the same calls succeed): 20000
+// of 301 rows 63.8 -> 29.7, of 511 rows 105.8 -> 40.2.  False, having launched
+// nothing, otherwise.
+template <typename T>
+static bool launch_lines16(const T *a, const T *b, const T *c, const T *d, T *out, int acc,
+                           const Lines &L, bool has_scratch, cudaStream_t st) {
+    if constexpr (!std::is_same<T, float>::value) {
+        return false;
+    } else {
+        if (L.stride != 1 || L.n <= MAX_SINGLE_PASS || L.n > 512) return false;
+        const bool vec = is_aligned16(a) && is_aligned16(c) && is_aligned16(d) &&
+                         is_aligned16(out) && (!b || is_aligned16(b)) && L.n % 4 == 0;
+        const int64_t blocks = (L.nsys + 3) / 4;
+        if (blocks >= (int64_t(1) << 31) || (!vec && !has_scratch)) return false;
+        if (vec)
+            k_lines<T, 16, 32><<<dim3(unsigned(blocks)), 128, 0, st>>>(a, b, c, d, out, acc,
+                                                                       L.nsys, L.n, 1);
+        else
+            k_lines_staged<T, 16, 32><<<dim3(unsigned(blocks)), 128, 0, st>>>(a, b, c, d, out, acc,
+                                                                              L.nsys, L.n);
+        return launch_ok();
+    }
+}
+
 template <typename T, int G>
 static void launch_lines(const T *a, const T *b, const T *c, const T *d, T *out, int acc,
                          const Lines &L, int vec_ok, cudaStream_t st) {
@@ -390,7 +420,7 @@ static void launch_strided(const T *a, const T *b, const T *c, const T *d, T *ou
             <<<strided_grid(L, SG), NT * SG, 0, st>>>(coef, d, out, L, L.nsys / L.inner);
 }
 
-// Contiguous FP32 systems of 256 < n <= 4096 through k_lines_tma with teams
+// Contiguous FP32 systems of 512 < n <= 4096 through k_lines_tma with teams
 // of TW warps, M rows per thread (n <= 32 * TW * M).  False, having launched nothing, when the
 // shared memory does not fit.
 template <int TW, int M, int SPS, bool SWZ = false>
@@ -465,7 +495,6 @@ static bool launch_lines_tma(const T *a, const T *b, const T *c, const T *d, T *
         // 8 rows per thread: one contiguous bulk copy per array and stage
         // (per-system swizzled 32-byte-row boxes measured slower at 1024 and
         // 2048 rows)
-        if (L.n <= 512) return launch_lines_tma_tw<2, 8, 8>(a, b, c, d, out, acc, L, st);
         if (L.n <= 1024) return launch_lines_tma_tw<4, 8, 4>(a, b, c, d, out, acc, L, st);
         if (L.n <= 2048) return launch_lines_tma_tw<8, 8, 2>(a, b, c, d, out, acc, L, st);
         // two teams of 8 warps, 16 rows per thread, taking one-system stages
@@ -743,11 +772,11 @@ static trid_status solve_lines(const T *a, const T *b, const T *c, const T *d, T
         }
         return cudaGetLastError() == cudaSuccess ? TRID_OK : TRID_ERR_CUDA;
     }
+    const bool has_scratch = ws != nullptr && ws_bytes >= long_ws_bytes<T>(L.nsys, L.n);
+    if (launch_lines16<T>(a, b, c, d, out, acc, L, has_scratch, st)) return TRID_OK;
     // up to 4096 contiguous FP32 rows: one pass, systems staged by bulk copies
     if (launch_lines_tma<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
-    if (launch_strided_tall<T>(a, b, c, d, out, acc, L, ws_bytes >= long_ws_bytes<T>(L.nsys, L.n),
-                               st))
-        return TRID_OK;
+    if (launch_strided_tall<T>(a, b, c, d, out, acc, L, has_scratch, st)) return TRID_OK;
     // strided FP32 up to 4096 rows: one cluster per strip of systems
     if (launch_chunk_cluster<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
     // long systems: tiled Thomas-PCR in passes

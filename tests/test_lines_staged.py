@@ -1,6 +1,6 @@
-"""Contiguous systems of up to 256 rows that are no whole 16-byte vectors,
-brought to shared memory element by element (k_lines_staged) or read directly
-(k_lines), against the FP64 oracle: lengths around every change of the lanes
+"""Contiguous systems of up to 256 rows (FP32: 512) that are no whole 16-byte
+vectors, brought to shared memory element by element (k_lines_staged) or read
+directly (k_lines), against the FP64 oracle: lengths around every change of the lanes
 per system, system counts that fill no warp or block, unaligned arrays, stored
 and accumulated, with values outside the systems that must not be used.  GPU
 only."""
@@ -58,3 +58,11 @@ def test_lengths(n, acc, dtype):
 def test_unaligned_arrays(n, dtype):
     for acc in (False, True):
         run(n, 70, dtype, acc, offset=1)
+
+
+@pytest.mark.parametrize("acc", [False, True], ids=["store", "acc"])
+@pytest.mark.parametrize("n", [257, 260, 271, 272, 300, 301, 384, 497, 508, 511, 512, 513, 516])
+def test_sixteen_rows_per_lane(n, acc):
+    for nsys in (1, 2, 5, 131):
+        run(n, nsys, np.float32, acc)
+    run(n, 9, np.float32, acc, offset=1)
