@@ -24,8 +24,8 @@
 //  k_lines_tma  contiguous FP32 systems of 512 < N <= 4096 in one pass:
 //             whole systems staged in shared memory by bulk copies, one team
 //             of warps per system (trid_lines_tma.cuh).
-//  k_team64   FP64 systems of 256 < N <= 4096 in one pass, a block per few
-//             neighbouring systems, 16 rows per thread (trid_team64.cuh).
+//  k_team   FP64 systems of 256 < N <= 4096 in one pass, a block per few
+//             neighbouring systems, 16 rows per thread (trid_team.cuh).
 //  k_twist    FP64 systems of N <= 256, when there are many: Thomas from both
 //             ends, two threads per system (trid_twist.cuh).
 //  k_chunk_cluster  strided FP32 systems of 256 < N <= 4096 in one pass:
@@ -36,7 +36,7 @@
 #include "trid_lines_tma.cuh"
 #include "trid_chunked.cuh"
 #include "trid_twist.cuh"
-#include "trid_team64.cuh"
+#include "trid_team.cuh"
 #include "../../include/trid.h"
 #include "trid_internal.h"
 
@@ -680,7 +680,7 @@ static bool launch_strided_tall(const T *a, const T *b, const T *c, const T *d, 
     }
 }
 
-// FP64 systems of 256 < n <= 4096 rows (strided: 3072) through k_team64.
+// FP64 systems of 256 < n <= 4096 rows (strided: 3072) through k_team.
 // Systems per block: the number that leaves the fewest of the block's threads
 // without a tile, blocks of up to 256 threads first (several share an SM and
 // hide each other's barriers), and of equal numbers the larger (strided rows
@@ -688,14 +688,29 @@ static bool launch_strided_tall(const T *a, const T *b, const T *c, const T *d, 
 // systems of 300 rows 86, 68, 64 us; 16000 of 512 rows 281, 268, 301; 10000 of
 // 700 rows 234, 239, 259; 3000 of 1400 rows 154, 156.  Strided systems of more
 // than 3072 rows would need more threads than registers allow for (4096 x 4096
-// 754 us against 706 in passes).  False, having launched nothing, when it does
-// not apply.
-template <int SG, int MODE>
-static bool launch_team64_form(const double *a, const double *b, const double *c, const double *d,
-                               double *out, int acc, const Lines &L, int tiles, cudaStream_t st) {
+// 754 us against 706 in passes).
+// FP32: what the single-pass paths before it do not take, that is contiguous
+// systems of more than 4096 rows (up to 8192: 512 tiles) or whose rows are no
+// 16-byte vectors, and strided ones whose rows are not.  Passes -> this: 3000
+// contiguous systems of 5000 rows 153 -> 53 us, 1500 of 8000 85 -> 55, 40 of 5000
+// 31 -> 7.4; unaligned, 1000 of 601 rows 20 -> 10.7, 10000 of 1001 107 -> 78, 1000
+// of 2047 29 -> 28; not unaligned beyond 4096, where a block's rows overflow the
+// L1 (2000 of 8191 167 -> 201).  Strided rows of 4 systems are half a sector,
+// whose other half the neighbouring block must find in the L2: up to 64 MiB in
+// all (61 systems of 1200 rows 22 -> 8.3 us, 1001 of 1500 25.6 -> 15.1; beyond it
+// 10001 of 2000 154 -> 278, 4001 of 1500 with accumulate 73 -> 124).  Of 2, a
+// quarter, only while the blocks fit the SMs at once (61 systems of 3000 rows
+// 22 -> 13; 4001 of 1500 with 2 per block 55 -> 64).  The rule itself looks
+// neither at out nor at accumulate.
+// False, having launched nothing, when it does not apply.
+constexpr int64_t TM_STRIDED_ROWS = (int64_t(64) << 20) / 20;   // five FP32 arrays
+
+template <typename T, int SG, int MODE>
+static bool launch_team_form(const T *a, const T *b, const T *c, const T *d, T *out, int acc,
+                             const Lines &L, int tiles, cudaStream_t st) {
     const int threads = (tiles * SG + 31) / 32 * 32;
-    const size_t smem = team64_smem(tiles, SG);
-    auto kern = k_team64<SG, MODE>;
+    const size_t smem = team_smem<T>(tiles, SG);
+    auto kern = k_team<T, SG, MODE>;
     if (kernel_blocks_per_sm(reinterpret_cast<const void *>(kern), threads, smem) < 1)
         return false;
     const int64_t blocks = (L.nsys + SG - 1) / SG;
@@ -705,38 +720,42 @@ static bool launch_team64_form(const double *a, const double *b, const double *c
 }
 
 template <typename T>
-static bool launch_team64(const T *a, const T *b, const T *c, const T *d, T *out, int acc,
-                          const Lines &L, cudaStream_t st) {
-    if constexpr (!std::is_same<T, double>::value) {
-        return false;
-    } else {
-        const DeviceInfo *di = device_info();
-        if (!di || !b || L.n > TM_M * TM_MAX_TILES || !strided_offsets_fit(L)) return false;
-        const int tiles = int((L.n + TM_M - 1) / TM_M);
-        const bool contig = L.stride == 1;
-        int sg = 0;
-        double best = 0.0;
-        for (int k = contig ? 1 : 2; k <= 8 && tiles * k <= TM_THREADS; k *= 2) {
-            if (sg && (L.nsys + k - 1) / k < 2 * di->sm_count) break;   // too few blocks
-            const int threads = (tiles * k + 31) / 32 * 32;
-            const double score = double(tiles * k) / threads -
-                                 (threads > 256 ? 0.2 : threads > 192 ? 0.03 : 0.0);
-            if (!sg || score >= best) { sg = k; best = score; }
-        }
-        auto al32 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; };
-        const bool vec = contig && L.n % 4 == 0 && al32(a) && al32(b) && al32(c) && al32(d) &&
-                         al32(out);
-#define TEAM64(S) (vec ? launch_team64_form<S, 1>(a, b, c, d, out, acc, L, tiles, st) \
-                       : launch_team64_form<S, 0>(a, b, c, d, out, acc, L, tiles, st))
-        switch (sg) {
-            case 1: return TEAM64(1);
-            case 2: return TEAM64(2);
-            case 4: return TEAM64(4);
-            case 8: return TEAM64(8);
-            default: return false;
-        }
-#undef TEAM64
+static bool launch_team(const T *a, const T *b, const T *c, const T *d, T *out, int acc,
+                        const Lines &L, cudaStream_t st) {
+    const DeviceInfo *di = device_info();
+    constexpr int THREADS = tm_threads<T>();
+    if (!di || !b || L.n > (sizeof(T) == 8 ? 4096 : 8192) || !strided_offsets_fit(L)) return false;
+    const int tiles = int((L.n + TM_M - 1) / TM_M);
+    const bool contig = L.stride == 1;
+    const bool vec = contig && (L.n * int64_t(sizeof(T))) % 16 == 0 && is_aligned16(a) &&
+                     is_aligned16(b) && is_aligned16(c) && is_aligned16(d);
+    int first = contig ? 1 : 2;
+    if (sizeof(T) == 4 && !contig) {
+        if (L.nsys * L.n > TM_STRIDED_ROWS) return false;
+        if (tiles * 4 <= THREADS) first = 4;
+        else if (L.nsys > 2 * int64_t(di->sm_count)) return false;
     }
+    if (sizeof(T) == 4 && contig && !vec && L.n > 4096) return false;
+    int sg = 0;
+    double best = 0.0;
+    for (int k = first; k <= 8 && tiles * k <= THREADS; k *= 2) {
+        if (sg && (L.nsys + k - 1) / k < 2 * di->sm_count) break;   // too few blocks
+        const int threads = (tiles * k + 31) / 32 * 32;
+        const double score = double(tiles * k) / threads -
+                             (threads > 256 ? 0.2 : threads > 192 ? 0.03 : 0.0);
+        if (!sg || score >= best) { sg = k; best = score; }
+    }
+    if (!sg) return false;
+#define TRID_TEAM(S) (vec ? launch_team_form<T, S, 1>(a, b, c, d, out, acc, L, tiles, st) \
+                          : launch_team_form<T, S, 0>(a, b, c, d, out, acc, L, tiles, st))
+    switch (sg) {
+        case 1: return TRID_TEAM(1);
+        case 2: return TRID_TEAM(2);
+        case 4: return TRID_TEAM(4);
+        case 8: return TRID_TEAM(8);
+        default: return false;
+    }
+#undef TRID_TEAM
 }
 
 template <typename T>
@@ -790,9 +809,9 @@ static trid_status solve_lines(const T *a, const T *b, const T *c, const T *d, T
     if (L.nsys * ntiles >= (int64_t(1) << 31) || L.nsys >= (int64_t(1) << 31))
         return TRID_ERR_UNSUPPORTED;
     if (ws_bytes < long_ws_bytes<T>(L.nsys, L.n) || ws == nullptr) return TRID_ERR_ALLOC;
-    // FP64 up to 4096 rows: one pass (it needs no scratch, but is taken only
-    // where the passes could run, so that the same calls succeed)
-    if (launch_team64<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
+    // FP64 up to 4096 rows, FP32 up to 8192: one pass (it needs no scratch, but is
+    // taken only where the passes could run, so that the same calls succeed)
+    if (launch_team<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
     T *ra = reinterpret_cast<T *>(ws);
     T *rc = reinterpret_cast<T *>(ws + one);
     T *rd = reinterpret_cast<T *>(ws + 2 * one);

@@ -1,4 +1,4 @@
-"""FP64 systems of 257 to 4096 rows in one pass (k_team64), against the FP64
+"""Systems of 257 to 4096 rows (FP32: 8192) in one pass (k_team), against the FP64
 oracle: row counts around every number of tiles per warp and every number of
 systems per block, contiguous in whole vectors and not, strided, system counts
 that fill no block, weakly coupled and nearly singular systems, and the limits
@@ -13,9 +13,9 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-def solve(dims, k, acc=False, offset=0, margin=None):
+def solve(dims, k, acc=False, offset=0, margin=None, dtype=np.float64, out_offset=None):
     n = int(np.prod(dims))
-    a, b, c, d = inputs.dominant_system((n,), seed=n + k, dtype=np.float64)
+    a, b, c, d = inputs.dominant_system((n,), seed=n + k, dtype=dtype)
     if margin is not None:
         b = np.abs(a) + np.abs(c) + margin
     idx = np.moveaxis(np.arange(n).reshape(dims[::-1]), len(dims) - 1 - k, 0)
@@ -23,13 +23,13 @@ def solve(dims, k, acc=False, offset=0, margin=None):
     a[idx[0].reshape(-1)] = np.nan     # not part of the system, so never used
     c[idx[-1].reshape(-1)] = np.nan
 
-    def dev(v):
-        t = torch.empty(n + offset, dtype=torch.float64, device="cuda")[offset:]
-        return t.copy_(torch.from_numpy(v))
+    def dev(v, offset=offset):
+        v = torch.from_numpy(v)
+        return torch.empty(n + offset, dtype=v.dtype, device="cuda")[offset:].copy_(v)
 
     ta, tb, tc, td = (dev(v) for v in (a, b, c, d))
-    u0 = inputs.random_rhs((n,), seed=5, dtype=np.float64) if acc else np.zeros(n)
-    tu = dev(u0) if acc else None
+    u0 = inputs.random_rhs((n,), seed=5, dtype=dtype) if acc else np.zeros(n, dtype)
+    tu = dev(u0, offset if out_offset is None else out_offset) if acc else None
     out = trid.solve(ta, tb, tc, td, dims, k, u=tu)
     if acc:
         assert np.array_equal(td.cpu().numpy(), d)
@@ -70,3 +70,26 @@ def test_weak_dominance(margin, tol):
     condition number (at most 3 / margin) times 2^-53, a few hundred times over."""
     check(*solve((1500, 9), 0, margin=margin), tol=tol)
     check(*solve((9, 1500), 1, margin=margin), tol=tol)
+
+
+@pytest.mark.parametrize("n", [513, 1023, 1025, 1537, 2049, 4095, 4097, 4100, 5000, 8176, 8191, 8192, 8193])
+@pytest.mark.parametrize("acc", [False, True], ids=["store", "acc"])
+def test_fp32(n, acc):
+    """The oracle in FP64 from the same FP32 arrays; 1e-5 of the largest value is
+    about 80 units of 2^-23, for a condition number of at most 3 and the sum."""
+    f = np.float32
+    check(*solve((n, 7), 0, acc, dtype=f), tol=1e-5)
+    check(*solve((n, 611), 0, acc, offset=1, dtype=f), tol=1e-5)
+    check(*solve((7, n), 1, acc, dtype=f), tol=1e-5)
+    check(*solve((307, n), 1, acc, dtype=f), tol=1e-5)
+
+
+def test_fp32_unaligned_out():
+    """Beyond 4096 rows the same kernel, so the same bits, as into an aligned
+    array; below, the aligned call runs another kernel and both are held to the
+    bound of test_fp32."""
+    f = np.float32
+    check(*solve((600, 40), 0, True, offset=0, dtype=f, out_offset=1), tol=1e-5)
+    got, ref = solve((5000, 40), 0, True, dtype=f, out_offset=1)
+    check(got, ref, tol=1e-5)
+    assert np.array_equal(got, solve((5000, 40), 0, True, dtype=f)[0])
