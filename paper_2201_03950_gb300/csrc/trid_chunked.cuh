@@ -304,13 +304,23 @@ k_chunk_cluster(const __grid_constant__ TmaSet maps, T *out, int accumulate, Lin
             }
         } else if (active) {
             T *ob = out + (int64_t(o) * L.inner * L.n + x);
+            // every load before the first store: out may not be reordered
+            // against itself, so a row at a time is a chain of round trips
+            // (4096 x 4096 along y with accumulate 215 -> 104 us)
+            if (accumulate) {
+                T ru[M];
+#pragma unroll
+                for (int k = 0; k < M; ++k) {
+                    const int gi = g0 + i0 + k;
+                    ru[k] = gi < n ? ob[int64_t(gi) * stride] : T(0);
+                }
+#pragma unroll
+                for (int k = 0; k < M; ++k) rd[k] += ru[k];
+            }
 #pragma unroll
             for (int k = 0; k < M; ++k) {
                 const int gi = g0 + i0 + k;
-                if (gi < n) {
-                    T *p = ob + int64_t(gi) * stride;
-                    *p = accumulate ? *p + rd[k] : rd[k];
-                }
+                if (gi < n) ob[int64_t(gi) * stride] = rd[k];
             }
         }
     }

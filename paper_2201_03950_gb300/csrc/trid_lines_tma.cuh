@@ -319,9 +319,16 @@ k_lines_tma(const __grid_constant__ TmaSet maps, const T *a, const T *b, const T
             }
             store_contig_vec<T, M>(o, rd);
         } else {
+            if (accumulate) {            // every load before the first store
+                T ru[M];
+#pragma unroll
+                for (int j = 0; j < M; ++j) ru[j] = i0 + j < n ? o[j] : T(0);
+#pragma unroll
+                for (int j = 0; j < M; ++j) rd[j] += ru[j];
+            }
 #pragma unroll
             for (int j = 0; j < M; ++j)
-                if (i0 + j < n) o[j] = accumulate ? o[j] + rd[j] : rd[j];
+                if (i0 + j < n) o[j] = rd[j];
         }
     }
 }

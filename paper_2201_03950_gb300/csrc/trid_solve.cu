@@ -8,24 +8,28 @@
 //             [g*M, g*M + M) loaded with 16-byte vector loads; the reduced
 //             system lives in registers and is solved with warp shuffles.
 //             No shared memory, no block-wide barrier: every warp runs
-//             independently.  Serves N <= 32*M.
+//             independently.  Serves N <= 32*M, and FP32 systems of up to
+//             512 rows with M = 16.  Systems that are no whole vectors are
+//             staged through shared memory (k_lines_staged).
 //  k_strided  systems strided in memory (y/z axes, and the reduced systems
 //             of the long path).  A block holds SG systems that are
 //             neighbours in memory (lane = system, so each row of the tile is
 //             one coalesced 128/256-byte segment) times NT tiles (thread
 //             group = tile); the reduced rows go through shared memory to a
-//             warp-shuffle solve with G = NT lanes per system.  N <= 32*M.
+//             warp-shuffle solve with G = NT lanes per system.  N <= 32*M,
+//             and FP32 systems of up to 1024 rows with M = 16, 24 or 32.
 //  k_long_*   longer systems: tiled Thomas-PCR in passes.  k_long_reduce
 //             writes the two reduced rows of each tile to scratch, the reduced
 //             systems (2 rows per tile) are solved by a recursive call, and
 //             k_long_subst recomputes each tile and substitutes the tile-end
 //             unknowns back.
-//             N <= 512 with 16 rows per lane (contiguous FP32).
 //  k_lines_tma  contiguous FP32 systems of 512 < N <= 4096 in one pass:
 //             whole systems staged in shared memory by bulk copies, one team
 //             of warps per system (trid_lines_tma.cuh).
-//  k_team   FP64 systems of 256 < N <= 4096 in one pass, a block per few
-//             neighbouring systems, 16 rows per thread (trid_team.cuh).
+//  k_team     FP64 systems of 256 < N <= 4096, and FP32 systems of up to 8192
+//             that neither k_lines_tma nor k_chunk_cluster can
+//             take, in one pass, a block per few neighbouring systems, 16 rows
+//             per thread (trid_team.cuh).
 //  k_twist    FP64 systems of N <= 256, when there are many: Thomas from both
 //             ends, two threads per system (trid_twist.cuh).
 //  k_chunk_cluster  strided FP32 systems of 256 < N <= 4096 in one pass:
@@ -107,13 +111,20 @@ k_lines(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ 
         }
         store_contig_vec<T, M>(out + base + i0, rd);
     } else {
+        if (accumulate) {                // every load before the first store
+            T ru[M];
+#pragma unroll
+            for (int j = 0; j < M; ++j) {
+                const int64_t i = i0 + j;
+                ru[j] = i < n && TRID_BOUNDS(base + i < nsys * n) ? out[base + i] : T(0);
+            }
+#pragma unroll
+            for (int j = 0; j < M; ++j) rd[j] += ru[j];
+        }
 #pragma unroll
         for (int j = 0; j < M; ++j) {
             const int64_t i = i0 + j;
-            if (i < n && TRID_BOUNDS(base + i < nsys * n)) {
-                if (accumulate) out[base + i] += rd[j];
-                else out[base + i] = rd[j];
-            }
+            if (i < n && TRID_BOUNDS(base + i < nsys * n)) out[base + i] = rd[j];
         }
     }
 }
@@ -321,15 +332,18 @@ k_long_subst(const T *__restrict__ a, const T *__restrict__ b, const T *__restri
         }
         store_contig_vec<T, M>(out + base + i0, rd);
     } else {
+        // every load before the first store (1000 systems of 9001 rows 133 -> 106 us)
+        if (accumulate) {
+            T ru[M];
 #pragma unroll
-        for (int j = 0; j < M; ++j) {
-            const int64_t i = i0 + j;
-            if (i < L.n) {
-                const int64_t p = base + i * L.stride;
-                if (accumulate) out[p] += rd[j];
-                else out[p] = rd[j];
-            }
+            for (int j = 0; j < M; ++j)
+                ru[j] = i0 + j < L.n ? out[base + (i0 + j) * L.stride] : T(0);
+#pragma unroll
+            for (int j = 0; j < M; ++j) rd[j] += ru[j];
         }
+#pragma unroll
+        for (int j = 0; j < M; ++j)
+            if (i0 + j < L.n) out[base + (i0 + j) * L.stride] = rd[j];
     }
 }
 

@@ -395,17 +395,29 @@ __device__ __forceinline__ void store_sys_tile(T *out, int accumulate, int64_t s
                                                const T (&rd)[VL_M]) {
     const int64_t p0 = s0 - pad + t * VL_M;
     const int64_t i0 = t * VL_M - pad;
-    if (i0 >= 0 && i0 + VL_M <= n && !accumulate) {
-        store_contig_vec<T, VL_M>(out + p0, rd);
+    T v[VL_M];
+    // accumulating: every load before the first store, in whole vectors (8192
+    // systems of 16 to 16384 rows, FP32 210 -> 131 us, FP64 1359 -> 1098 with the plain second pass)
+    if (i0 >= 0 && i0 + VL_M <= n) {
+        if (accumulate) {
+            load_contig_vec<T, VL_M>(out + p0, v);
+#pragma unroll
+            for (int j = 0; j < VL_M; ++j) v[j] += rd[j];
+            store_contig_vec<T, VL_M>(out + p0, v);
+        } else {
+            store_contig_vec<T, VL_M>(out + p0, rd);
+        }
         return;
     }
 #pragma unroll
     for (int j = 0; j < VL_M; ++j) {
         const int64_t i = i0 + j;
-        if (i >= 0 && i < n) {
-            if (accumulate) out[p0 + j] += rd[j];
-            else out[p0 + j] = rd[j];
-        }
+        v[j] = accumulate && i >= 0 && i < n ? out[p0 + j] : T(0);
+    }
+#pragma unroll
+    for (int j = 0; j < VL_M; ++j) {
+        const int64_t i = i0 + j;
+        if (i >= 0 && i < n) out[p0 + j] = accumulate ? v[j] + rd[j] : rd[j];
     }
 }
 
