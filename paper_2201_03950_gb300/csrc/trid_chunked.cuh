@@ -215,7 +215,12 @@ k_chunk_cluster(const __grid_constant__ TmaSet maps, T *out, int accumulate, Lin
                 ra[k] = T(0); rb[k] = T(1); rc[k] = T(0); rd[k] = T(0);
             }
         }
-        __syncthreads();  // the box is free: fetch the next strip's behind this one
+        // The box is free: fetch the next strip's behind this one.  The reads above
+        // are generic accesses and the copy writes through the async proxy, which
+        // a block barrier alone does not order: without the fence a copy of a
+        // strip found in the L2 overtook the last reads of a busy SM.
+        fence_proxy_async_smem();
+        __syncthreads();
         if (tid == 0 && ok && strip + ncl < nstrips) issue(strip + ncl);
 
         T as, cs, ds, ae, ce, de;

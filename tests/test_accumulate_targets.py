@@ -47,3 +47,18 @@ def test_mesh(dtype, dims, k, offset):
     u = dev(u0, offset)
     trid.solve(dev(a), dev(b), dev(c), dev(d), dims, k, u=u)
     check(u, u0, oracle.solve_mesh(a, b, c, d, dims, k), dtype)
+
+
+@pytest.mark.parametrize("dims", [(8192, 512), (3000, 1400), (4096, 2048)])
+def test_clusters_many_strips(dims):
+    """Several strips of systems per cluster, ten times: the copy of a strip must
+    not overtake the reads of the strip before it."""
+    n = int(np.prod(dims))
+    a, b, c, d = inputs.dominant_system((n,), seed=11, dtype=np.float32)
+    u0 = inputs.random_rhs((n,), seed=12, dtype=np.float32)
+    ref = oracle.solve_mesh(a, b, c, d, dims, 1)
+    ta, tb, tc, td = (dev(v) for v in (a, b, c, d))
+    for _ in range(10):
+        u = dev(u0)
+        trid.solve(ta, tb, tc, td, dims, 1, u=u)
+        check(u, u0, ref, np.float32)
