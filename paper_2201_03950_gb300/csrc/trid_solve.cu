@@ -644,9 +644,10 @@ static bool launch_twist(const T *a, const T *b, const T *c, const T *d, T *out,
 //   512 rows   1024 systems 3.7 against 5.7 us, 4096 10.5 / 12.3, 8192 23.2 / 19.5
 //   768 rows   1024 systems 4.7 / 6.7, 4864 17.9 / 19.5, 8192 31.8 / 28.0
 //   1024 rows  256 systems 5.6 / 5.5, 1024 5.6 / 7.2, 4096 23.0 / 20.0
-// and accumulating, where the clusters store without TMA,
-//   512 rows   4096 systems 11.7 / 20.8;  768 rows  4864 systems 31.0 / 35.4
-//   1024 rows  1024 systems 5.3 / 9.4, 2048 25.1 / 20.5 (16 systems a block spill)
+// and accumulating, where the clusters store without TMA (a call through the
+// binding takes about 8 us),
+//   512 rows   4096 systems 8.0 / 14.2;  768 rows  4864 systems 22.7 / 24.7
+//   1024 rows  1024 systems 8.0 / 9.6 (16 systems a block spill)
 // The choice is the same for storing and accumulating and whatever `out` is: a
 // differentiable ADI recomputes with stored solves the states that its forward
 // accumulated, and must get the same bits.  Arrays that the clusters do not
@@ -655,14 +656,26 @@ template <int M, int SG>
 static bool launch_strided_tall_form(const float *a, const float *b, const float *c,
                                      const float *d, float *out, int acc, const Lines &L,
                                      cudaStream_t st) {
-    ArrayCoef<float> coef{a, b, c};
-    if (acc)
-        k_strided<float, M, 32, SG, true, ArrayCoef<float>>
-            <<<strided_grid(L, SG), 32 * SG, 0, st>>>(coef, d, out, L, L.nsys / L.inner);
-    else
-        k_strided<float, M, 32, SG, false, ArrayCoef<float>>
-            <<<strided_grid(L, SG), 32 * SG, 0, st>>>(coef, d, out, L, L.nsys / L.inner);
-    return launch_ok();
+    // chained to the previous kernel by programmatic dependent launch (50 steps of
+    // a 1024 x 1024 differentiable ADI, called directly: forward 670 -> 586 us; as
+    // graphs, without the attribute, the plain pointers alone: forward 587 -> 566,
+    // backward 1924 -> 1886)
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = strided_grid(L, SG);
+    cfg.blockDim = dim3(32 * SG);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl_launch_allowed(st) ? 1 : 0;
+    const PlainCoef<float> coef{a, b, c};
+    auto kern = acc ? k_strided<float, M, 32, SG, true, PlainCoef<float>>
+                    : k_strided<float, M, 32, SG, false, PlainCoef<float>>;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, coef, d, out, L, L.nsys / L.inner);
+    note_cuda_error(e);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
 }
 
 template <typename T>

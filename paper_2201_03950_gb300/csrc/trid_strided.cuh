@@ -23,10 +23,28 @@ template <typename T> struct SysCfg;
 template <> struct SysCfg<float> { static constexpr int SG = 16; };
 template <> struct SysCfg<double> { static constexpr int SG = 16; };
 
+// As ArrayCoef below, for kernels launched with programmatic dependent launch:
+// without __restrict__, so that no load is moved ahead of the grid-dependency
+// wait.
+template <typename T>
+struct PlainCoef {
+    static constexpr bool PDL = true;
+    const T *a, *b, *c;
+    __device__ __forceinline__ PlainCoef shifted(int64_t base) const {
+        return PlainCoef{a + base, b + base, c + base};
+    }
+    __device__ __forceinline__ void get(int off, int i, int n, T &ra, T &rb, T &rc) const {
+        ra = (i == 0) ? T(0) : a[off];
+        rb = b[off];
+        rc = (i == n - 1) ? T(0) : c[off];
+    }
+};
+
 // Coefficients read from arrays; a of row 0 and c of row n-1 are not read.
 // b == nullptr means unit diagonal (the reduced systems of the long path).
 template <typename T>
 struct ArrayCoef {
+    static constexpr bool PDL = false;
     const T *__restrict__ a;
     const T *__restrict__ b;
     const T *__restrict__ c;
@@ -54,6 +72,7 @@ struct ArrayCoef {
 // Dirichlet boundary nodes.
 template <typename T>
 struct AdiCoef {
+    static constexpr bool PDL = false;
     T lam;
     __device__ __forceinline__ AdiCoef shifted(int64_t) const { return *this; }
     __device__ __forceinline__ void get(int, int i, int n, T &ra, T &rb, T &rc) const {
@@ -93,6 +112,10 @@ k_strided(Coef coef, const T *d, T *out, Lines L, int64_t outer) {
 
     const int64_t o = int64_t(blockIdx.z) * gridDim.y + blockIdx.y;
     if (o >= outer) return;  // whole block: no barrier is skipped by part of it
+    if constexpr (Coef::PDL) {
+        pdl_trigger();
+        pdl_wait();
+    }
     {
         const bool active = x < L.inner;
         const int64_t base = active ? x + o * L.inner * L.n : 0;
