@@ -116,13 +116,15 @@ const char *trid_last_cuda_error(void);
  * are solved in one pass too, without scratch, when their arrays start on
  * 16-byte boundaries and (contiguous systems) the length is a multiple of 4
  * or (strided systems) the contiguous extent times 4 bytes is a multiple of
- * 16: whole systems staged in shared memory, or one thread-block cluster per
- * strip of 16 systems.  All other long systems (longer, FP64, unaligned) go
- * through the hybrid in several passes, which need scratch of
- * trid_solve_workspace_bytes(...) bytes; this entry point takes it from a
+ * 16: a warp or a team of warps per system, or one block or thread-block
+ * cluster per strip of neighbouring systems.  All other long systems (longer,
+ * FP64, unaligned) need scratch of trid_solve_workspace_bytes(...) bytes.  With
+ * it, those of up to 4096 rows (contiguous FP32 in 16-byte vectors: 8192) are
+ * mostly still solved in one pass, which leaves the scratch untouched; the rest
+ * go through the hybrid in several passes.  This entry point takes it from a
  * library-owned pool of the current device, grown (device synchronisation,
- * cudaFree, cudaMalloc) only when the multi-pass path is taken and the pool
- * is too small: such a call must not be inside a stream capture (pre-size
+ * cudaFree, cudaMalloc) only when such a system comes and the pool is too
+ * small: such a call must not be inside a stream capture (pre-size
  * the pool with trid_init to avoid it).  The pool is one buffer per device,
  * shared by every stream: multi-pass calls whose work overlaps on the GPU
  * (different streams, no ordering between them) race on it and may return
