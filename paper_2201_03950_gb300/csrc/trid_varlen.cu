@@ -534,7 +534,7 @@ struct VItem {
 };
 
 __device__ __forceinline__ VItem vitem_fetch(unsigned long long *ctr, int64_t limit, int64_t base,
-                                             const longlong2 *__restrict__ meta) {
+                                             const longlong2 *meta) {
     VItem v;
     v.item = (long long)atomicAdd(ctr, 1ull);
     v.s0 = 0;
@@ -547,11 +547,15 @@ __device__ __forceinline__ VItem vitem_fetch(unsigned long long *ctr, int64_t li
     return v;
 }
 
+// meta and work are plain pointers: k_varlen_plan1 may still be writing them when
+// this kernel starts (trid_tma.cuh).  a, b and c are not: the plan is launched
+// without the attribute, so what wrote them has completed before it starts, and
+// no kernel writes them while this one runs.
 template <typename T, int VL_M>
 __global__ void __launch_bounds__(VL_THREADS, (sizeof(T) == 4 && VL_M == 8) ? 2 : 1)
 k_varlen_solve(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ c, const T *d,
                T *out, int accumulate, int64_t nsys, int64_t total, int64_t max_len,
-               VarlenWork *work, const longlong2 *__restrict__ meta, int nlevels, int *status,
+               VarlenWork *work, const longlong2 *meta, int nlevels, int *status,
                int e1, int e2, int team_threads) {
     constexpr int VL_M2_N = vl_m2_n(VL_M), VL_SHORT_N = vl_short_n(VL_M);
     const int64_t m1_max = vl_class_max(e1, VL_M), m2_max = vl_class_max(e2, VL_M);

@@ -23,13 +23,14 @@ def test_system_counts(nsys):
     lens[rng.integers(0, nsys)] = 5000
     off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
     a, b, c, d = inputs.dominant_system((int(off[-1]),), seed=nsys, dtype=np.float32)
-    ref = oracle.solve_varlen(a, b, c, d, off)
     t = [torch.from_numpy(v).cuda() for v in (a, b, c, d)]
     ws = torch.full((trid.varlen_workspace_bytes(nsys),), 255, dtype=torch.uint8, device="cuda")
-    toff = torch.from_numpy(off).cuda()
-    for _ in range(2):      # the second call finds the first one's plan in the workspace
+    # the second and third call find the plan of another division of the same rows
+    # in the workspace
+    for o in (off, np.concatenate([[0], np.cumsum(lens[::-1])]).astype(np.int64), off):
+        ref = oracle.solve_varlen(a, b, c, d, o)
         x = t[3].clone()
-        trid.solve_varlen(*t[:3], x, toff, int(lens.max()), workspace=ws)
+        trid.solve_varlen(*t[:3], x, torch.from_numpy(o).cuda(), int(lens.max()), workspace=ws)
         assert np.max(np.abs(x.cpu().numpy() - ref)) <= 1e-5 * np.max(np.abs(ref))
     assert trid.device_status() == 0
 
