@@ -7,7 +7,9 @@
 #include <atomic>
 #include <cstdlib>
 #include <cstring>
+#include <iterator>
 #include <mutex>
+#include <unordered_map>
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -51,39 +53,82 @@ const DeviceInfo *device_info() {
 }
 
 namespace {
-struct OccEntry {
-    const void *kernel;
-    int dev, threads;
-    size_t smem;
-    int blocks;
-};
-constexpr int kOccCache = 256;
-OccEntry g_occ[kOccCache];
-int g_nocc = 0;
-}  // namespace
-
-namespace {
-struct ClusterEntry {
+// Results of the launch queries, kept per (kernel, device, cluster size, threads,
+// dynamic shared memory).  Several kernels' shared memory follows the extents, so
+// a process that meets many sizes asks many keys: a hash table, emptied if it
+// ever holds kLaunchCacheMax.
+struct LaunchKey {
     const void *kernel;
     int dev, csize, threads;
     size_t smem;
-    int clusters;
+    bool operator==(const LaunchKey &o) const {
+        return kernel == o.kernel && dev == o.dev && csize == o.csize && threads == o.threads &&
+               smem == o.smem;
+    }
 };
-constexpr int kClusterCache = 64;
-ClusterEntry g_ccache[kClusterCache];
-int g_ncc = 0;
+struct LaunchKeyHash {
+    size_t operator()(const LaunchKey &k) const {
+        uint64_t h = uint64_t(reinterpret_cast<uintptr_t>(k.kernel));
+        const uint64_t rest[2] = {uint64_t(k.dev) << 40 | uint64_t(k.csize) << 20 |
+                                      uint64_t(k.threads), uint64_t(k.smem)};
+        for (uint64_t v : rest) h = (h ^ v) * 0x9e3779b97f4a7c15ull, h ^= h >> 29;
+        return size_t(h);
+    }
+};
+using LaunchCache = std::unordered_map<LaunchKey, int, LaunchKeyHash>;
+constexpr size_t kLaunchCacheMax = 1 << 16;
+LaunchCache g_occ;      // blocks per SM (csize 0)
+LaunchCache g_ccache;   // resident clusters
+LaunchCache g_limit;    // dynamic shared memory allowed (threads, csize, smem 0)
+
+bool launch_find(const LaunchCache &c, const LaunchKey &k, int &v) {
+    const auto it = c.find(k);
+    if (it == c.end()) return false;
+    v = it->second;
+    return true;
+}
+void launch_keep(LaunchCache &c, const LaunchKey &k, int v) {
+    try {
+        if (c.size() >= kLaunchCacheMax) c.clear();
+        c.emplace(k, v);
+    } catch (...) {   // no memory: asked again next time
+    }
+}
+void launch_forget(LaunchCache &c, int dev) {
+    for (auto it = c.begin(); it != c.end();)
+        it = it->first.dev == dev ? c.erase(it) : std::next(it);
+}
+
+// The dynamic shared memory that launches of `kernel` may ask for.  The limit is
+// an attribute of the function, shared by every thread of the process: it is
+// raised once, to all that a block can have, so that no query for a small size
+// takes it away between another thread's query and launch.
+bool raise_smem_limit(const void *kernel, int dev, int max_optin, int &limit) {
+    const LaunchKey key{kernel, dev, 0, 0, 0};
+    if (launch_find(g_limit, key, limit)) return true;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    if (e == cudaSuccess) {
+        limit = max_optin - int(fa.sharedSizeBytes);
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        note_cuda_error(e);
+        return false;
+    }
+    launch_keep(g_limit, key, limit);
+    return true;
+}
 }  // namespace
 
 int cluster_capacity(const void *kernel, int csize, int threads, size_t smem) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (int i = 0; i < g_ncc; ++i) {
-        const ClusterEntry &e = g_ccache[i];
-        if (e.kernel == kernel && e.dev == dev && e.csize == csize && e.threads == threads &&
-            e.smem == smem)
-            return e.clusters;
-    }
+    const LaunchKey key{kernel, dev, csize, threads, smem};
+    int n = 0;
+    if (launch_find(g_ccache, key, n)) return n;
     if (csize > 8) {
         const cudaError_t ae =
             cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -104,48 +149,34 @@ int cluster_capacity(const void *kernel, int csize, int threads, size_t smem) {
     cfg.dynamicSmemBytes = smem;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int n = 0;
     const cudaError_t oe = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
     if (oe != cudaSuccess) {
         cudaGetLastError();
         n = 0;
     }
-    if (g_ncc < kClusterCache)
-        g_ccache[g_ncc++] = ClusterEntry{kernel, dev, csize, threads, smem, n};
+    launch_keep(g_ccache, key, n);
     return n;
 }
 
 int kernel_blocks_per_sm(const void *kernel, int threads, size_t smem) {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const DeviceInfo *di = device_info();
+    if (!di || cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (int i = 0; i < g_nocc; ++i) {
-        const OccEntry &e = g_occ[i];
-        if (e.kernel == kernel && e.dev == dev && e.threads == threads && e.smem == smem)
-            return e.blocks;
-    }
-    // The attribute is per function: raise it to the largest size this
-    // function is ever queried with, never lower it (a cached smaller query
-    // must not shrink the limit a larger launch relies on).
-    int need = int(smem);
-    for (int i = 0; i < g_nocc; ++i)
-        if (g_occ[i].kernel == kernel && g_occ[i].dev == dev && int(g_occ[i].smem) > need)
-            need = int(g_occ[i].smem);
-    const cudaError_t ae =
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, need);
-    if (ae != cudaSuccess) {
-        cudaGetLastError();
-        note_cuda_error(ae);
-        return 0;
-    }
-    int blocks = 0;
-    const cudaError_t oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, threads, smem);
+    const LaunchKey key{kernel, dev, 0, threads, smem};
+    int blocks = 0, limit = 0;
+    if (launch_find(g_occ, key, blocks)) return blocks;
+    if (!raise_smem_limit(kernel, dev, di->max_smem_optin, limit)) return 0;
+    const cudaError_t oe =
+        smem > size_t(limit) ? cudaErrorInvalidValue
+                             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel,
+                                                                             threads, smem);
     if (oe != cudaSuccess) {
         cudaGetLastError();
         note_cuda_error(oe);
         return 0;
     }
-    if (g_nocc < kOccCache) g_occ[g_nocc++] = OccEntry{kernel, dev, threads, smem, blocks};
+    launch_keep(g_occ, key, blocks);
     return blocks;
 }
 
@@ -248,14 +279,9 @@ static void forget_device(int dev) {
     g_info_ok[dev] = false;
     if (g_aux_stream[dev]) cudaStreamDestroy(g_aux_stream[dev]);
     g_aux_stream[dev] = nullptr;
-    int k = 0;
-    for (int i = 0; i < g_nocc; ++i)
-        if (g_occ[i].dev != dev) g_occ[k++] = g_occ[i];
-    g_nocc = k;
-    k = 0;
-    for (int i = 0; i < g_ncc; ++i)
-        if (g_ccache[i].dev != dev) g_ccache[k++] = g_ccache[i];
-    g_ncc = k;
+    launch_forget(g_occ, dev);
+    launch_forget(g_ccache, dev);
+    launch_forget(g_limit, dev);
 }
 
 cudaStream_t aux_stream() {
