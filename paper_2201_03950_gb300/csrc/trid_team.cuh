@@ -94,7 +94,8 @@ k_team(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ c
     }
     for (int s = 1; s < tiles; s <<= 1) {
         if (on) { ra0[t] = fa; rc0[t] = fc; rd0[t] = fd; }
-        const bool big = fmax(fabs(fa), fabs(fc)) >= negligible;
+        // (a coupling that is no number counts: it goes on to the whole system)
+        const bool big = !(fmax(fabs(fa), fabs(fc)) < negligible);
         if (!__syncthreads_or(big)) break;
         if (on) {
             const bool lo = tile >= s, hi = tile + s < tiles;

@@ -93,3 +93,19 @@ def test_fp32_unaligned_out():
     got, ref = solve((5000, 40), 0, True, dtype=f, out_offset=1)
     check(got, ref, tol=1e-5)
     assert np.array_equal(got, solve((5000, 40), 0, True, dtype=f)[0])
+
+
+@pytest.mark.parametrize("which", ["a", "b", "c"])
+@pytest.mark.parametrize("dims,k,dtype", [((3000, 5), 0, np.float64), ((5, 3000), 1, np.float64),
+                                          ((700, 9), 0, np.float64), ((5000, 3), 0, np.float32),
+                                          ((1001, 5), 0, np.float32), ((41, 1500), 1, np.float32)])
+def test_a_coefficient_that_is_no_number_spoils_its_whole_system(dims, k, dtype, which):
+    """And no other one, as in the passes: no value of it is determined."""
+    n = int(np.prod(dims))
+    v = dict(zip("abcd", inputs.dominant_system((n,), seed=1, dtype=dtype)))
+    idx = np.moveaxis(np.arange(n).reshape(dims[::-1]), len(dims) - 1 - k, 0)
+    v[which][idx[dims[k] // 2, 2]] = np.nan
+    t = [torch.from_numpy(x).cuda() for x in v.values()]
+    x = trid.solve(*t, dims, k).cpu().numpy()[idx]
+    assert np.all(np.isnan(x[:, 2]))
+    assert np.all(np.isfinite(np.delete(x, 2, axis=1)))
