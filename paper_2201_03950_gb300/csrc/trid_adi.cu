@@ -671,10 +671,20 @@ static trid_status adi_dims(const int64_t *dims, int ndim, int64_t (&n3)[3], int
     return TRID_OK;
 }
 
-// Planes of up to 32 x 32 points: the whole-plane schedule before the windowed
-// one (72 meshes of 32^3: 13.6 against 15.5 us a step, one mesh 5.4 against
-// 7.4; 80 x 32 x 32, 72 meshes: 30.0 against 24.6).
-static bool adi_small_planes(const int64_t *n3) { return n3[0] <= 32 && n3[1] <= 32; }
+// Whether the whole-plane schedule goes before the windowed one: planes of up to
+// 32 x 32 points, and not too many of them.  A step, windowed against whole
+// planes, at 32 x 32: 32^3, one mesh 7.3 against 5.1 us, 72 15.5 / 12.8, 200 25.8
+// / 25.7, 400 46.8 / 57.0; 64 deep, 32 meshes 14.7 / 13.7, 72 21.1 / 23.1; 96 deep,
+// one mesh 7.5 / 6.7, 8 12.4 / 13.8; 128 deep, one mesh 7.7 / 7.9.  At 16 x 32: 72
+// meshes 160 deep 31.0 / 30.1, 192 deep 35.3 / 40.6, 400 of 32 deep 34.4 / 30.9.
+// (One mesh of more than 160 planes, which the whole-plane schedule declines:
+// 32 x 32 x 192 windowed 8.7, two-pass 15.4; 24 x 32 x 192 8.0, general 24.7.)
+static bool adi_planes_before_window(const int64_t *n3, int64_t nb) {
+    if (n3[0] > 32 || n3[1] > 32) return false;
+    const int64_t planes = n3[2] * nb;
+    if (n3[0] <= 16) return planes <= 12800;
+    return planes <= (n3[2] <= 32 ? 6400 : n3[2] <= 80 ? 2100 : n3[2] <= 96 ? 100 : 0);
+}
 
 // nb meshes stacked along z through the whole-plane schedule, where it is the
 // faster one: not for few, long z lines (pass B has a thread per half line;
@@ -698,8 +708,26 @@ trid_status adi3_planes_run(void *u, int64_t nb, const int64_t *n3, double lam, 
                           st, taken);
 }
 
+// nb meshes stacked along z through the windowed or the whole-plane schedule,
+// each where it applies and is the faster one; `taken` is false, and nothing
+// launched, when neither takes them.
+trid_status adi3_stack_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
+                           trid_dtype dtype, void *ws, cudaStream_t st, bool &taken) {
+    taken = false;
+    trid_status s = TRID_OK;
+    const bool planes_first = dtype == TRID_F64 || adi_planes_before_window(n3, nb);
+    if (planes_first) s = adi3_planes_run(u, nb, n3, lam, nsteps, dtype, ws, st, taken);
+    if (!taken && s == TRID_OK && dtype == TRID_F32)
+        s = adi_run_window(static_cast<float *>(u), n3, lam, nsteps, static_cast<char *>(ws), st,
+                           nb, taken);
+    if (!taken && s == TRID_OK && !planes_first)
+        s = adi3_planes_run(u, nb, n3, lam, nsteps, dtype, ws, st, taken);
+    return s;
+}
+
 // Batches of 3D meshes stacked along z (each mesh keeps its own boundary
-// planes), through the two-pass schedule; used by adi_step_batched.
+// planes) through the first of the windowed, whole-plane and two-pass schedules
+// that suits them; used by adi_step_batched where the two-pass one applies.
 bool adi3_batch_eligible(const int64_t *n3, int ndim) { return adi2_eligible(n3, ndim); }
 
 size_t adi3_batch_ws_bytes(const int64_t *n3, size_t esz, int64_t nb) {
@@ -713,11 +741,7 @@ trid_status adi3_batch_run(void *u, int64_t nb, const int64_t *n3, double lam, i
     if ((reinterpret_cast<uintptr_t>(ws) % 256) != 0) return TRID_ERR_MISALIGNED;
     if (!is_aligned16(u)) return TRID_ERR_MISALIGNED;
     bool taken = false;
-    trid_status s = TRID_OK;
-    if (dtype == TRID_F32 && !adi_small_planes(n3))
-        s = adi_run_window(static_cast<float *>(u), n3, lam, nsteps, static_cast<char *>(ws), st,
-                           nb, taken);
-    if (!taken && s == TRID_OK) s = adi3_planes_run(u, nb, n3, lam, nsteps, dtype, ws, st, taken);
+    const trid_status s = adi3_stack_run(u, nb, n3, lam, nsteps, dtype, ws, st, taken);
     if (taken || s != TRID_OK) return s;
     if (dtype == TRID_F32)
         return adi_run_2pass<float>(static_cast<float *>(u), n3, float(lam), nsteps,
@@ -763,11 +787,7 @@ extern "C" trid_status adi_step(void *u, const int64_t *dims, int ndim, double l
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (ndim == 3) {
         bool taken = false;
-        if (dtype == TRID_F32 && !adi_small_planes(n3))
-            s = adi_run_window(static_cast<float *>(u), n3, lambda, nsteps,
-                               static_cast<char *>(workspace), st, 1, taken);
-        if (!taken && s == TRID_OK)
-            s = adi3_planes_run(u, 1, n3, lambda, nsteps, dtype, workspace, st, taken);
+        s = adi3_stack_run(u, 1, n3, lambda, nsteps, dtype, workspace, st, taken);
         if (taken || s != TRID_OK) return s;
     }
     if (adi2_eligible(n3, ndim) && is_aligned16(u)) {

@@ -74,6 +74,10 @@ int *device_status_word();
 trid_status adi3_planes_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
                             trid_dtype dtype, void *ws, cudaStream_t st, bool &taken);
 
+// The same through the windowed or the whole-plane schedule.
+trid_status adi3_stack_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
+                           trid_dtype dtype, void *ws, cudaStream_t st, bool &taken);
+
 // 3D ADI on a batch of meshes stacked along z (windowed, whole-plane and
 // two-pass schedules).
 bool adi3_batch_eligible(const int64_t *n3, int ndim);
