@@ -348,11 +348,14 @@ trid_status trid_varlen_autotune(const void *a, const void *b, const void *c, co
  * 3D meshes run stacked along z through the kernels of the 3D step, and the
  * rest go through adi_step one after another.  `workspace` (256-byte aligned)
  * should hold adi_batched_workspace_bytes(nbatch, dims, ndim, dtype) bytes.
- * It must do so when every extent is a multiple of 16 and z is at least 32;
- * other 3D meshes are also stepped with less, as many at a time as it holds:
- * the least is the scratch of one mesh (adi_workspace_bytes), and none
- * (workspace NULL) where a mesh can be resident on chip.  Errors as adi_step;
- * asynchronous on `stream`.
+ * It must do so when every extent is a multiple of 16 and z is at least 32 (the
+ * whole batch's scratch); for other 3D meshes those are at most 2 GiB, and they
+ * are also stepped with less, as many at a time as it holds: the least is the
+ * scratch of one mesh (adi_workspace_bytes), and none (workspace NULL) where a
+ * mesh can be resident on chip.  A mesh's result does not depend on its place in
+ * the batch, nor on the size of the scratch (with none at all, or less than a
+ * resident mesh, it may differ by rounding).  Errors as adi_step; asynchronous
+ * on `stream`.
  */
 size_t adi_batched_workspace_bytes(int64_t nbatch, const int64_t *dims, int ndim,
                                    trid_dtype dtype);

@@ -691,15 +691,16 @@ static bool adi_planes_before_window(const int64_t *n3, int64_t nb) {
 // 31 x 40 x 200, one mesh: 17.8 against 14.6 us a step), nor in FP64 for
 // planes that leave half of the SMs without one when the two-pass schedule,
 // which cuts planes into tiles, can run (64^3, one mesh: 43.6 against 39.1;
-// 80^3 43.4 against 67.8).  `taken` is false, and nothing launched, otherwise.
-trid_status adi3_planes_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
-                            trid_dtype dtype, void *ws, cudaStream_t st, bool &taken) {
+// 80^3 43.4 against 67.8).  The rule looks at the whole batch of `all` meshes, of
+// which these may be a group.  `taken` is false, and nothing launched, otherwise.
+trid_status adi3_planes_run(void *u, int64_t nb, int64_t all, const int64_t *n3, double lam,
+                            int nsteps, trid_dtype dtype, void *ws, cudaStream_t st, bool &taken) {
     taken = false;
     const DeviceInfo *di = device_info();
     if (!di || n3[2] < 3) return TRID_OK;
-    if (n3[2] > 160 && n3[0] * n3[1] * nb < 2048) return TRID_OK;
+    if (n3[2] > 160 && n3[0] * n3[1] * all < 2048) return TRID_OK;
     if (dtype == TRID_F64 && adi2_eligible(n3, 3) && n3[0] * n3[1] >= 4096 &&
-        nb * (n3[2] - 2) * 2 < di->sm_count)
+        all * (n3[2] - 2) * 2 < di->sm_count)
         return TRID_OK;
     if (dtype == TRID_F32)
         return adi_planes_run(static_cast<float *>(u), static_cast<float *>(ws), n3, nb, lam,
@@ -709,19 +710,20 @@ trid_status adi3_planes_run(void *u, int64_t nb, const int64_t *n3, double lam, 
 }
 
 // nb meshes stacked along z through the windowed or the whole-plane schedule,
-// each where it applies and is the faster one; `taken` is false, and nothing
-// launched, when neither takes them.
-trid_status adi3_stack_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
-                           trid_dtype dtype, void *ws, cudaStream_t st, bool &taken) {
+// each where it applies and is the faster one for the batch of `all` meshes that
+// they are a group of; `taken` is false, and nothing launched, when neither takes
+// them.
+trid_status adi3_stack_run(void *u, int64_t nb, int64_t all, const int64_t *n3, double lam,
+                           int nsteps, trid_dtype dtype, void *ws, cudaStream_t st, bool &taken) {
     taken = false;
     trid_status s = TRID_OK;
-    const bool planes_first = dtype == TRID_F64 || adi_planes_before_window(n3, nb);
-    if (planes_first) s = adi3_planes_run(u, nb, n3, lam, nsteps, dtype, ws, st, taken);
+    const bool planes_first = dtype == TRID_F64 || adi_planes_before_window(n3, all);
+    if (planes_first) s = adi3_planes_run(u, nb, all, n3, lam, nsteps, dtype, ws, st, taken);
     if (!taken && s == TRID_OK && dtype == TRID_F32)
         s = adi_run_window(static_cast<float *>(u), n3, lam, nsteps, static_cast<char *>(ws), st,
                            nb, taken);
     if (!taken && s == TRID_OK && !planes_first)
-        s = adi3_planes_run(u, nb, n3, lam, nsteps, dtype, ws, st, taken);
+        s = adi3_planes_run(u, nb, all, n3, lam, nsteps, dtype, ws, st, taken);
     return s;
 }
 
@@ -741,7 +743,7 @@ trid_status adi3_batch_run(void *u, int64_t nb, const int64_t *n3, double lam, i
     if ((reinterpret_cast<uintptr_t>(ws) % 256) != 0) return TRID_ERR_MISALIGNED;
     if (!is_aligned16(u)) return TRID_ERR_MISALIGNED;
     bool taken = false;
-    const trid_status s = adi3_stack_run(u, nb, n3, lam, nsteps, dtype, ws, st, taken);
+    const trid_status s = adi3_stack_run(u, nb, nb, n3, lam, nsteps, dtype, ws, st, taken);
     if (taken || s != TRID_OK) return s;
     if (dtype == TRID_F32)
         return adi_run_2pass<float>(static_cast<float *>(u), n3, float(lam), nsteps,
@@ -787,7 +789,7 @@ extern "C" trid_status adi_step(void *u, const int64_t *dims, int ndim, double l
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (ndim == 3) {
         bool taken = false;
-        s = adi3_stack_run(u, 1, n3, lambda, nsteps, dtype, workspace, st, taken);
+        s = adi3_stack_run(u, 1, 1, n3, lambda, nsteps, dtype, workspace, st, taken);
         if (taken || s != TRID_OK) return s;
     }
     if (adi2_eligible(n3, ndim) && is_aligned16(u)) {

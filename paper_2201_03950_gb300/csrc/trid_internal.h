@@ -68,15 +68,15 @@ trid_status solve_with_scratch(const void *a, const void *b, const void *c, void
 // trid_get_device_status); kernels that run bounded waits record failures there.
 int *device_status_word();
 
-// 3D ADI on nb meshes stacked along z through the whole-plane schedule, where it
-// is the fastest one (else `taken` is false and nothing is launched); ws holds
-// nb meshes.
-trid_status adi3_planes_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
-                            trid_dtype dtype, void *ws, cudaStream_t st, bool &taken);
+// 3D ADI on nb meshes stacked along z, a group of a batch of `all`, through the
+// whole-plane schedule, where it is the fastest one for the batch (else `taken` is
+// false and nothing is launched); ws holds nb meshes.
+trid_status adi3_planes_run(void *u, int64_t nb, int64_t all, const int64_t *n3, double lam,
+                            int nsteps, trid_dtype dtype, void *ws, cudaStream_t st, bool &taken);
 
 // The same through the windowed or the whole-plane schedule.
-trid_status adi3_stack_run(void *u, int64_t nb, const int64_t *n3, double lam, int nsteps,
-                           trid_dtype dtype, void *ws, cudaStream_t st, bool &taken);
+trid_status adi3_stack_run(void *u, int64_t nb, int64_t all, const int64_t *n3, double lam,
+                           int nsteps, trid_dtype dtype, void *ws, cudaStream_t st, bool &taken);
 
 // 3D ADI on a batch of meshes stacked along z (windowed, whole-plane and
 // two-pass schedules).

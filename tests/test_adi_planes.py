@@ -119,6 +119,41 @@ def test_too_little_scratch_is_refused():
     assert st == 5   # TRID_ERR_ALLOC
 
 
+def test_scratch_asked_for_is_bounded():
+    dc, nd = trid._dims((100, 100, 100))
+    one = trid.adi_workspace_bytes((100, 100, 100), "float32")
+    for nb in (1, 60, 500, 600, 1000, 1 << 20):
+        need = int(trid.load().adi_batched_workspace_bytes(nb, dc, nd, trid.TRID_F32))
+        assert one <= need <= 2 << 30
+
+
+@pytest.mark.parametrize("dims,dtype", [((30, 31, 170), np.float32), ((33, 29, 20), np.float64),
+                                        ((25, 28, 24), np.float32)])
+def test_place_and_scratch_do_not_change_the_bits(dims, dtype):
+    """Five times the same mesh, with scratch for one to five of them."""
+    nb = 5
+    u0 = np.tile(field(dims, 1, 5, dtype), nb)
+    mesh = int(np.prod(dims)) * np.dtype(dtype).itemsize
+    least = trid.adi_workspace_bytes(dims, "float32" if dtype is np.float32 else "float64")
+    first = None
+    for size in (None, least, 2 * mesh, 3 * mesh, 4 * mesh):
+        if size is not None and size < least:
+            continue
+        st, got, _ = stepped(u0, nb, dims, 0.25, 3, ws_bytes=size)
+        assert st == 0
+        first = got[:got.size // nb] if first is None else first
+        assert np.array_equal(got, np.tile(first, nb))
+
+
+def test_less_than_one_meshs_scratch_is_refused():
+    dims = (50, 51, 40)     # too large to be resident on chip
+    u0 = field(dims, 2, 5, np.float32)
+    least = trid.adi_workspace_bytes(dims, "float32")
+    for size in (u0.nbytes // 2, least - 256):
+        st, got, _ = stepped(u0, 2, dims, 0.25, 3, ws_bytes=size)
+        assert st == 5 and np.array_equal(got, u0)   # TRID_ERR_ALLOC
+
+
 def test_box_edges_do_not_enter():
     dims = (34, 29, 31)
     u0 = field(dims, 1, 8, np.float32).reshape(dims[::-1])
