@@ -709,6 +709,12 @@ trid_status adi3_planes_run(void *u, int64_t nb, int64_t all, const int64_t *n3,
                           st, taken);
 }
 
+// Whether the windowed schedule takes meshes of these extents.
+bool adi3_window_suits(const int64_t *n3, double lam) {
+    static thread_local AdiWPlan p;
+    return adiw_plan(n3, 1, lam, p);
+}
+
 // nb meshes stacked along z through the windowed or the whole-plane schedule,
 // each where it applies and is the faster one for the batch of `all` meshes that
 // they are a group of; `taken` is false, and nothing launched, when neither takes

@@ -74,7 +74,8 @@ int *device_status_word();
 trid_status adi3_planes_run(void *u, int64_t nb, int64_t all, const int64_t *n3, double lam,
                             int nsteps, trid_dtype dtype, void *ws, cudaStream_t st, bool &taken);
 
-// The same through the windowed or the whole-plane schedule.
+// The same through the windowed (FP32) or the whole-plane schedule.
+bool adi3_window_suits(const int64_t *n3, double lam);
 trid_status adi3_stack_run(void *u, int64_t nb, int64_t all, const int64_t *n3, double lam,
                            int nsteps, trid_dtype dtype, void *ws, cudaStream_t st, bool &taken);
 

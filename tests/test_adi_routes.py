@@ -45,7 +45,11 @@ CASES = [((24, 32, 192), SINGLE, 0.1, F4, "k_adi_xyw"), ((32, 32, 256), SINGLE, 
          ((32, 32, 128), 20, 0.1, F4, "k_adi_xyw"), ((32, 32, 48), 60, 0.1, F4, "k_adi_xyw"),
          ((32, 32, 32), SINGLE, 0.1, F4, "k_adi_planes"), ((32, 32, 32), 72, 0.1, F4, "k_adi_planes"),
          ((16, 32, 160), SINGLE, 0.1, F4, "k_adi_planes"),
-         ((32, 32, 128), SINGLE, 0.3, F4, "k_adi_planes")]      # not windowed: slow decay
+         ((32, 32, 128), SINGLE, 0.3, F4, "k_adi_planes"),      # not windowed: slow decay
+         # extents that are no multiples of 16, stacked: windowed too
+         ((40, 64, 64), 1, 0.1, F4, "k_adi_xyw"), ((120, 96, 96), 3, 0.1, F4, "k_adi_xyw"),
+         ((104, 128, 16), 5, 0.1, F4, "k_adi_xyw"), ((40, 64, 64), 3, 0.3, F4, "k_adi_planes"),
+         ((40, 32, 16), 3, 0.1, F4, "k_adi_planes")]
 
 
 @pytest.mark.parametrize("dims,nb,lam,dtype,kernel", CASES,
