@@ -246,11 +246,18 @@ using namespace trid;
 // faster, given scratch: in FP32 from 2048 points on (24^3: 24 meshes 18.5 ->
 // 9.7 us a step, 1000 meshes 128 -> 78; 16^3, 72 meshes: 12.0 -> 7.7; 8^3, 1000
 // meshes: 9.8 against 11.2), but not many meshes much longer along x than along
-// y, whose short columns fill few lanes (64 x 16 x 16, 1000 meshes: 76 against
-// 88; 67 x 16 x 17, 8 meshes: 14.9 -> 7.1).  In FP64 k_adi_fused is as fast or
-// faster (16^3, 72 meshes: 30 against 38; 8^3, 1000: 28 against 47).
+// y, whose short columns fill few lanes: there k_adi_fused steps up to one mesh
+// per SM in the time of one, and whole planes are faster while the meshes are
+// few for their y z extent.  Fitted to 123 extents of 32 to 160 by 3 to 32 by 3 to
+// 24 with 1 to 150 meshes (the choice is 0.6% slower than the better one on the
+// mean): 160 x 8 x 8, 24 meshes 8.8 -> 8.2, 72 meshes 8.8 against 10.7, 150 9.3
+// against 18.6; 64 x 16 x 16, 72 meshes 1.56 times as fast, 1000: 76 against 88.
+// In FP64 k_adi_fused is as fast or faster (16^3, 72 meshes: 30 against 38; 8^3,
+// 1000: 28 against 47).
 static bool ba_planes_first(const int64_t *n3, size_t esz, int64_t nb) {
-    return esz == 4 && n3[0] * n3[1] * n3[2] >= 2048 && (nb <= 300 || n3[0] <= 2 * n3[1]);
+    if (esz != 4 || n3[0] * n3[1] * n3[2] < 2048) return false;
+    return n3[0] <= 2 * n3[1] ||
+           (nb <= 300 && 5 * nb <= (n3[0] <= 48 ? 4 : 3) * n3[1] * n3[2]);
 }
 
 // Meshes stacked at a time: all, or where their scratch would pass 2 GiB, as few

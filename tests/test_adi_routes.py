@@ -49,7 +49,10 @@ CASES = [((24, 32, 192), SINGLE, 0.1, F4, "k_adi_xyw"), ((32, 32, 256), SINGLE, 
          # extents that are no multiples of 16, stacked: windowed too
          ((40, 64, 64), 1, 0.1, F4, "k_adi_xyw"), ((120, 96, 96), 3, 0.1, F4, "k_adi_xyw"),
          ((104, 128, 16), 5, 0.1, F4, "k_adi_xyw"), ((40, 64, 64), 3, 0.3, F4, "k_adi_planes"),
-         ((40, 32, 16), 3, 0.1, F4, "k_adi_planes")]
+         ((40, 32, 16), 3, 0.1, F4, "k_adi_planes"),
+         # long rows, short columns: whole planes for few meshes only
+         ((160, 8, 8), 8, 0.2, F4, "k_adi_planes"), ((160, 8, 8), 72, 0.2, F4, "k_adi_fused"),
+         ((64, 8, 8), 150, 0.2, F4, "k_adi_fused"), ((64, 16, 16), 72, 0.2, F4, "k_adi_planes")]
 
 
 @pytest.mark.parametrize("dims,nb,lam,dtype,kernel", CASES,
