@@ -593,12 +593,18 @@ static bool launch_chunk_cluster(const T *a, const T *b, const T *c, const T *d,
 
 // FP64 systems of up to 256 rows through k_twist, when there are enough of
 // them: its time does not fall below the latency of one system's two chains
-// (256 rows: 53 us strided, 65 us contiguous, for any number of systems up to
-// about 9700), where the tiled kernels take 0.0125 us (strided) and 0.012 us
-// (contiguous) per 256-row system, both in proportion to the rows: the times
-// cross at 4096 strided (53 against 51 us) and about 6000 contiguous systems
-// (6144 of 128 rows: 35 against 38 us).  At 65536 systems of 256 rows they
-// are 305 against 655 us (strided) and 381 against 596 us (contiguous).
+// (256 rows: 53 us strided, 62 accumulating, 66 to 70 contiguous, for any number
+// of systems up to about 9700), where the tiled kernels' grows by rounds: a round of
+// 32 strided systems per SM takes 47 us at 256 rows, 25 at 128, 14 at 64, against 53,
+// 29 and 16 of this kernel.  Strided systems come here from the second round on
+// (4868 systems on 152 SMs: 53 against 74 us at 256 rows, 29 / 35, 16 / 21), a little
+// earlier where the first is no faster (8 rows 6.1 against 8.2, 192 rows, tiles for
+// 256, 41 / 45); contiguous ones, whose rounds are shorter, at about 6000 (256 rows: 68
+// against 66 us there, 70 against 78 at 7400; 192 rows 53 against 65).  At 65536
+// systems of 256 rows they are 305 against 655 us (strided) and 381 against 596 us
+// (contiguous).  Accumulating, d' fills the shared memory too: beyond 232 rows an SM
+// holds three warps, and a round of 48 systems per SM takes 1.27 rounds of the tiled
+// kernel (7400 systems of 256 rows 119 against 94 us, 15000 180 / 170).
 // Contiguous systems only when their halves are whole 32-byte vectors (with
 // scalar loads 378 us against 402 us at 43571 systems of 201 rows, and slower
 // than that at two warps per block), and not when accumulating (d' then
@@ -623,14 +629,22 @@ static bool launch_twist(const T *a, const T *b, const T *c, const T *d, T *out,
     if constexpr (!std::is_same<T, double>::value) {
         return false;
     } else {
-        if (!b || L.n > MAX_SINGLE_PASS || !strided_offsets_fit(L)) return false;
+        const DeviceInfo *di = device_info();
+        if (!di || !b || L.n > MAX_SINGLE_PASS || !strided_offsets_fit(L)) return false;
+        const int64_t sms = di->sm_count;
         if (L.stride == 1) {
             auto al32 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; };
             return L.nsys >= 6144 && !acc && L.n % 4 == 0 && al32(a) && al32(b) && al32(c) &&
                    al32(d) && al32(out) &&
                    launch_twist_form<false, true, 2>(a, b, c, d, out, L, st);
         }
-        if (L.nsys < 4608) return false;
+        const bool early = L.n <= 24 || (L.n > 128 && L.n <= 192);
+        if (L.nsys <= (early ? 30 : 32) * sms) return false;
+        if (acc) {
+            const int64_t warps = di->smem_per_sm / (twist_smem(int(L.n), false, true, 1) + 1024);
+            const int64_t rounds = (L.nsys - 1) / (TW_SYS * (warps > 0 ? warps : 1) * sms) + 1;
+            if (warps < 4 && 14 * rounds > 10 * ((L.nsys - 1) / (32 * sms) + 1)) return false;
+        }
         return acc ? launch_twist_form<true, false, 1>(a, b, c, d, out, L, st)
                    : launch_twist_form<false, false, 1>(a, b, c, d, out, L, st);
     }

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
+from graphs import graph_text
 from paper_2201_03950_gb300 import inputs, trid
 
 torch = pytest.importorskip("torch")
@@ -25,18 +26,6 @@ def scratch(dims, nb, dtype):
     need = (trid.adi_workspace_bytes(dims, dtype) if nb is None else
             int(trid.load().adi_batched_workspace_bytes(nb, dc, nd, trid._code(dtype))))
     return torch.empty(need, dtype=torch.uint8, device="cuda") if need else None
-
-
-def graph_of(u, dims, nb, lam, steps, ws, path):
-    """The captured call as text."""
-    step(u.clone(), dims, nb, lam, steps, ws)      # the library's per-device set-up
-    torch.cuda.synchronize()
-    g = torch.cuda.CUDAGraph(keep_graph=True)
-    g.enable_debug_mode()
-    with torch.cuda.graph(g):
-        step(u, dims, nb, lam, steps, ws)
-    g.debug_dump(str(path))
-    return path.read_text()
 
 
 SINGLE, F4, F8 = None, np.float32, np.float64
@@ -70,7 +59,8 @@ def test_route(dims, nb, lam, dtype, kernel, tmp_path):
     ws = scratch(dims, nb, u.dtype)
     # (the route of FP64 meshes on chip depends on there being 8 steps)
     steps = 8 if len(dims) == 2 else 2
-    assert kernel in graph_of(u.clone(), dims, nb, lam, steps, ws, tmp_path / "graph.dot")
+    v = u.clone()
+    assert kernel in graph_text(lambda: step(v, dims, nb, lam, steps, ws), tmp_path / "graph.dot")
     step(u, dims, nb, lam, 2, ws)
     got = u.cpu().numpy()
     for b in {0, (nb or 1) - 1}:

@@ -1,0 +1,52 @@
+"""Which kernel solves a mesh's systems, read from a captured graph, at the sizes
+where a slower one must not be chosen; and the solution there against the FP64
+oracle.  GPU only."""
+import numpy as np
+import pytest
+
+import oracle
+from graphs import graph_text
+from paper_2201_03950_gb300 import inputs, trid
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu, pytest.mark.filterwarnings("ignore:DEBUG")]
+
+TOL = {np.float32: 1e-5, np.float64: 1e-12}
+
+
+def check(dims, k, dtype, acc, kernel, path, offset=0):
+    n = int(np.prod(dims))
+    host = inputs.dominant_system((n,), seed=n, dtype=dtype)
+    dev = [torch.empty(n + offset, dtype=torch.from_numpy(v).dtype, device="cuda")[offset:]
+           .copy_(torch.from_numpy(v)) for v in host]
+    u = torch.zeros_like(dev[3]) if acc else None
+    x = dev[3].clone()
+    got = trid.solve(*dev[:3], x, dims, k, u=u).cpu().numpy()
+    ref = oracle.solve_mesh(*host, dims, k)
+    assert np.max(np.abs(got - ref)) <= TOL[dtype] * np.max(np.abs(ref))
+    assert kernel in graph_text(lambda: trid.solve(*dev[:3], x, dims, k, u=u), path / "graph.dot")
+
+
+@pytest.mark.parametrize("n", [64, 128, 256])
+@pytest.mark.parametrize("acc", [False, True], ids=["store", "acc"])
+def test_fp64_short_strided(n, acc, tmp_path):
+    """Two threads per system from the second round of the tiled kernel on."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    check((32 * sms, n), 1, np.float64, acc, "k_strided", tmp_path)
+    check((32 * sms + 4, n), 1, np.float64, acc, "k_twist", tmp_path)
+
+
+@pytest.mark.parametrize("n", [8, 192])
+def test_fp64_short_strided_early(n, tmp_path):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    check((30 * sms, n), 1, np.float64, False, "k_strided", tmp_path)
+    check((30 * sms + 4, n), 1, np.float64, False, "k_twist", tmp_path)
+
+
+def test_fp64_accumulating_rounds(tmp_path):
+    """256 rows: a round of 48 systems per SM against rounds of 32."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    check((48 * sms + 4, 256), 1, np.float64, True, "k_strided", tmp_path)
+    check((48 * sms + 4, 256), 1, np.float64, False, "k_twist", tmp_path)
+    check((48 * sms + 4, 200), 1, np.float64, True, "k_twist", tmp_path)
+    check((64 * sms + 4, 256), 1, np.float64, True, "k_twist", tmp_path)
