@@ -57,9 +57,8 @@ constexpr int MAX_SINGLE_PASS = 32 * TILE_M;  // longest system served in one pa
 // Contiguous systems: one group of G lanes per system.
 // ---------------------------------------------------------------------------
 template <typename T, int M, int G>
-__global__ void __launch_bounds__(256)
-k_lines(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ c, const T *d,
-        T *out, int accumulate, int64_t nsys, int64_t n, int vec_ok) {
+__device__ __forceinline__ void lines_body(const T *a, const T *b, const T *c, const T *d, T *out,
+                                           int accumulate, int64_t nsys, int64_t n, int vec_ok) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int g = lane % G;
@@ -127,6 +126,24 @@ k_lines(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ 
             if (i < n && TRID_BOUNDS(base + i < nsys * n)) out[base + i] = rd[j];
         }
     }
+}
+
+template <typename T, int M, int G>
+__global__ void __launch_bounds__(256)
+k_lines(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ c, const T *d,
+        T *out, int accumulate, int64_t nsys, int64_t n, int vec_ok) {
+    lines_body<T, M, G>(a, b, c, d, out, accumulate, nsys, n, vec_ok);
+}
+
+// The same, launched while the previous kernel of the stream drains: plain
+// pointers, so that no load is moved ahead of the wait.
+template <typename T, int M, int G>
+__global__ void __launch_bounds__(128)
+k_lines_chained(const T *a, const T *b, const T *c, const T *d, T *out, int accumulate,
+                int64_t nsys, int64_t n, int vec_ok) {
+    pdl_trigger();
+    pdl_wait();
+    lines_body<T, M, G>(a, b, c, d, out, accumulate, nsys, n, vec_ok);
 }
 
 // Contiguous systems whose rows are no whole 16-byte vectors (a length or an
@@ -372,7 +389,9 @@ static size_t long_ws_bytes(int64_t nsys, int64_t n) {
 // lane.  Teams of two warps fed by bulk copies, which took them before, pay a
 // named barrier and a reduced solve in shared memory per system; that -> this:
 // 8192 systems of 300 rows 17.7 -> 11.6 us, of 512 rows 18.3 -> 14.5, 30000 of 512
-// rows 50.7 -> 44.9 (accumulating 70.5 -> 53.7), 1024 of 512 rows 4.1 -> 3.1.
+// rows 50.7 -> 44.9 (accumulating 70.5 -> 53.7).  Chained to the previous kernel by
+// programmatic dependent launch, as those are: one call after another, without
+// it, 1000 systems of 400 rows took 6.1 us where the teams took 3.9.
 // Systems that are no whole 16-byte vectors went through scratch in passes (and
 // are taken only where those could run, so that the same calls succeed): 20000
 // of 301 rows 63.8 -> 29.7, of 511 rows 105.8 -> 40.2.  False, having launched
@@ -388,12 +407,24 @@ static bool launch_lines16(const T *a, const T *b, const T *c, const T *d, T *ou
                          is_aligned16(out) && (!b || is_aligned16(b)) && L.n % 4 == 0;
         const int64_t blocks = (L.nsys + 3) / 4;
         if (blocks >= (int64_t(1) << 31) || (!vec && !has_scratch)) return false;
-        if (vec)
-            k_lines<T, 16, 32><<<dim3(unsigned(blocks)), 128, 0, st>>>(a, b, c, d, out, acc,
-                                                                       L.nsys, L.n, 1);
-        else
-            k_lines_staged<T, 16, 32><<<dim3(unsigned(blocks)), 128, 0, st>>>(a, b, c, d, out, acc,
-                                                                              L.nsys, L.n);
+        if (vec) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.gridDim = dim3(unsigned(blocks));
+            cfg.blockDim = dim3(128);
+            cfg.stream = st;
+            cfg.attrs = attr;
+            cfg.numAttrs = pdl_launch_allowed(st) ? 1 : 0;
+            const cudaError_t e = cudaLaunchKernelEx(&cfg, k_lines_chained<T, 16, 32>, a, b, c, d,
+                                                     out, acc, L.nsys, L.n, 1);
+            note_cuda_error(e);
+            if (e != cudaSuccess) cudaGetLastError();
+            return e == cudaSuccess;
+        }
+        k_lines_staged<T, 16, 32><<<dim3(unsigned(blocks)), 128, 0, st>>>(a, b, c, d, out, acc,
+                                                                          L.nsys, L.n);
         return launch_ok();
     }
 }

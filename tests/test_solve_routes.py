@@ -50,3 +50,28 @@ def test_fp64_accumulating_rounds(tmp_path):
     check((48 * sms + 4, 256), 1, np.float64, False, "k_twist", tmp_path)
     check((48 * sms + 4, 200), 1, np.float64, True, "k_twist", tmp_path)
     check((64 * sms + 4, 256), 1, np.float64, True, "k_twist", tmp_path)
+
+
+@pytest.mark.parametrize("acc", [False, True], ids=["store", "acc"])
+def test_fp32_contiguous_257_to_512(acc, tmp_path):
+    check((400, 1000), 0, np.float32, acc, "k_lines_chained", tmp_path)
+
+
+@pytest.mark.parametrize("n,nsys", [(260, 1), (400, 64), (512, 1000)])
+def test_chained_calls_see_each_other(n, nsys):
+    """Ten calls in a row, each on what the one before has written, as with a
+    synchronisation in between."""
+    t = [torch.from_numpy(v).cuda() for v in inputs.dominant_system((n * nsys,), seed=n, dtype=np.float32)]
+    out = []
+    for wait in (False, True):
+        x, b, u = t[3].clone(), t[1].clone(), torch.zeros_like(t[3])
+        for _ in range(10):
+            trid.solve(t[0], b, t[2], x, (n, nsys), 0)
+            if wait:
+                torch.cuda.synchronize()
+            trid.solve(t[0], b, t[2], x, (n, nsys), 0, u=u)
+            if wait:
+                torch.cuda.synchronize()
+            torch.add(t[1], u.abs(), out=b)     # the next call's coefficients
+        out.append((x, u))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
