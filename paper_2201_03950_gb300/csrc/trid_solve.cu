@@ -156,10 +156,12 @@ k_lines_chained(const T *a, const T *b, const T *c, const T *d, T *out, int accu
 // every one touches up to 32 sectors, eight times over.  FP32, that kernel ->
 // this one: 43571 systems of 201 rows 49.3 -> 37.0 us, accumulating 94.7 -> 41.7;
 // 90000 of 101 rows 40.7 -> 40.1 and 96.7 -> 44.6; 160000 of 17 rows 13.8 -> 16.4
-// and 38.0 -> 16.4; 250000 of 7 rows 13.9 -> 8.9 (FP64 is bound by its
-// arithmetic in both).  So it is taken when accumulating and for one, two or
-// 32 lanes per system; otherwise the lines of a warp meet in few enough
-// sectors.
+// and 38.0 -> 16.4; 300000 of 16 rows (unaligned arrays) 26.8 -> 20.8, of 8 rows 16.5
+// -> 12.4, but of 3 rows 7.0 -> 8.2, of 13 16.4 -> 19.3 (FP64 is bound by its
+// arithmetic in both, and gains at few systems: 1000 of 3 rows 12.3 -> 8.2).  So it is
+// taken when accumulating, for 32 lanes per system, and for one or two lanes in
+// FP64 and where the lines start 32 or 64 bytes apart; otherwise the lines of a
+// warp meet in few enough sectors.
 __device__ __forceinline__ int ls_pad(int q) { return q + (q >> 3); }
 template <typename T>
 __device__ __forceinline__ void ls_copy(T *dst, const T *src) {
@@ -434,7 +436,8 @@ static void launch_lines(const T *a, const T *b, const T *c, const T *d, T *out,
                          const Lines &L, int vec_ok, cudaStream_t st) {
     const int64_t warps = (L.nsys + (32 / G) - 1) / (32 / G);
     const int64_t blocks = (warps + 7) / 8;
-    if (vec_ok || !(acc || G <= 2 || G == 32))
+    const bool shorts = G <= 2 && (sizeof(T) == 8 || L.n % 8 == 0);
+    if (vec_ok || !(acc || shorts || G == 32))
         k_lines<T, TILE_M, G><<<dim3(unsigned(blocks)), 256, 0, st>>>(a, b, c, d, out, acc,
                                                                        L.nsys, L.n, vec_ok);
     else

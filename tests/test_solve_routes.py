@@ -24,7 +24,9 @@ def check(dims, k, dtype, acc, kernel, path, offset=0):
     got = trid.solve(*dev[:3], x, dims, k, u=u).cpu().numpy()
     ref = oracle.solve_mesh(*host, dims, k)
     assert np.max(np.abs(got - ref)) <= TOL[dtype] * np.max(np.abs(ref))
-    assert kernel in graph_text(lambda: trid.solve(*dev[:3], x, dims, k, u=u), path / "graph.dot")
+    text = graph_text(lambda: trid.solve(*dev[:3], x, dims, k, u=u), path / "graph.dot")
+    assert kernel in text
+    return text
 
 
 @pytest.mark.parametrize("n", [64, 128, 256])
@@ -75,3 +77,13 @@ def test_chained_calls_see_each_other(n, nsys):
             torch.add(t[1], u.abs(), out=b)     # the next call's coefficients
         out.append((x, u))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("n,dtype,acc,offset,kernel", [
+    (3, np.float32, False, 0, "k_lines"), (13, np.float32, False, 0, "k_lines"),
+    (8, np.float32, False, 1, "k_lines_staged"), (16, np.float32, False, 1, "k_lines_staged"),
+    (3, np.float32, True, 0, "k_lines_staged"), (3, np.float64, False, 0, "k_lines_staged"),
+    (201, np.float32, False, 0, "k_lines_staged")])
+def test_contiguous_no_whole_vectors(n, dtype, acc, offset, kernel, tmp_path):
+    text = check((n, 5000), 0, dtype, acc, kernel, tmp_path, offset)
+    assert ("staged" in kernel) == ("staged" in text)
