@@ -258,11 +258,14 @@ static void launch_adj_strided(const T *a, const T *b, const T *c, const T *x, c
     // then touches all pages of the nine arrays, and rows of 128 bytes instead
     // of 64 halve the touches.  FP32: 512 x 512 x 64 along z (64 MiB a system)
     // 172 -> 94 us, 256^3 along z (64 MiB) 136 -> 116, but 256 x 256 x 128 along z
-    // (32 MiB) 53.1 against 53.6 and 256^3 along y (256 KiB) 100 against 112.
+    // (32 MiB) 53.1 against 53.6 and 256^3 along y (256 KiB) 100 against 112.  The
+    // line: 48 MiB, 128 rows 97 -> 78, 32 rows 99 -> 72, 16 rows 86 -> 71, but 256 rows
+    // 84 -> 87 there and 112 -> 101 at 56 MiB.
     // Bringing the arrays by TMA boxes as the solves do took 118 and 139 us
     // along z and 112 along y: five boxes leave room for one stage per block.
     if constexpr (sizeof(T) == 4) {
-        if (L.n * L.stride * int64_t(sizeof(T)) >= (int64_t(48) << 20)) {
+        const int64_t mib = L.n > 128 ? 51 : 48;
+        if (L.n * L.stride * int64_t(sizeof(T)) >= (mib << 20)) {
             k_adjoint_strided<T, ADJ_M, NT, 32><<<strided_grid(L, 32), NT * 32, 0, st>>>(
                 a, b, c, x, gx, ga, gb, gc, gd, L, L.nsys / L.inner);
             return;

@@ -6,18 +6,20 @@ import numpy as np
 import pytest
 
 import oracle
+from graphs import graph_text
 from paper_2201_03950_gb300 import trid
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-SPAN = (48 << 20) // 4   # elements
+def span(n):   # elements
+    return ((51 if n > 128 else 48) << 20) // 4
 
 
 @pytest.mark.parametrize("n", [3, 8, 9, 17, 40, 100, 256])
 @pytest.mark.parametrize("below", [False, True], ids=["wide", "narrower"])
 def test_sampled_systems(n, below):
-    inner = SPAN // n - 1 if below else SPAN // n + 5
+    inner = span(n) // n - 1 if below else span(n) // n + 5
     dims = (inner, n)
     g = torch.Generator(device="cuda").manual_seed(n)
 
@@ -36,3 +38,12 @@ def test_sampled_systems(n, below):
         ref = oracle.adjoint(*(np.ascontiguousarray(v[:, k], dtype=np.float64) for v in cols[:5]))
         for r, v in zip(ref, cols[5:]):
             assert np.max(np.abs(v[:, k] - r)) <= 2e-5 * max(np.max(np.abs(r)), 1e-30)
+
+
+@pytest.mark.filterwarnings("ignore:DEBUG")
+@pytest.mark.parametrize("n,mib,threads", [(256, 50, 512), (256, 52, 1024), (128, 49, 512), (128, 47, 256)])
+def test_systems_per_block(n, mib, threads, tmp_path):
+    inner = (mib << 20) // 4 // n
+    t = [torch.rand(inner * n, device="cuda") + 2 * (k == 1) for k in range(5)]
+    text = graph_text(lambda: trid.adjoint(*t, (inner, n), 1), tmp_path / "graph.dot")
+    assert f",{threads},0\\>" in text
