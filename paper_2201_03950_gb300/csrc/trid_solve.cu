@@ -866,26 +866,27 @@ static trid_status solve_lines(const T *a, const T *b, const T *c, const T *d, T
         }
         return cudaGetLastError() == cudaSuccess ? TRID_OK : TRID_ERR_CUDA;
     }
-    const bool has_scratch = ws != nullptr && ws_bytes >= long_ws_bytes<T>(L.nsys, L.n);
+    // long systems: tiled Thomas-PCR in passes, within the limits of the grid and of
+    // the kernels' 32-bit thread and line indices; the one-pass kernels that take
+    // over from them are used only where those could run, so that the same calls succeed
+    const int64_t ntiles = (L.n + TILE_M - 1) / TILE_M;
+    const bool passes = (contig || (ntiles + 7) / 8 <= 65535) &&
+                        L.nsys * ntiles < (int64_t(1) << 31) && L.nsys < (int64_t(1) << 31);
+    const bool has_scratch =
+        passes && ws != nullptr && ws_bytes >= long_ws_bytes<T>(L.nsys, L.n);
     if (launch_lines16<T>(a, b, c, d, out, acc, L, has_scratch, st)) return TRID_OK;
     // up to 4096 contiguous FP32 rows: one pass, systems staged by bulk copies
     if (launch_lines_tma<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
     if (launch_strided_tall<T>(a, b, c, d, out, acc, L, has_scratch, st)) return TRID_OK;
     // strided FP32 up to 4096 rows: one cluster per strip of systems
     if (launch_chunk_cluster<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
-    // long systems: tiled Thomas-PCR in passes
-    const int64_t ntiles = (L.n + TILE_M - 1) / TILE_M;
+    // (a problem no path serves reports TRID_ERR_UNSUPPORTED whether or not scratch
+    // was given)
+    if (!passes) return TRID_ERR_UNSUPPORTED;
+    if (!has_scratch) return TRID_ERR_ALLOC;
     const int64_t R = 2 * ntiles;
     const size_t one = align_up(size_t(L.nsys) * size_t(R) * sizeof(T), 256);
-    // limits of the multi-pass path first, so that a problem no path serves
-    // reports TRID_ERR_UNSUPPORTED whether or not scratch was given
-    if (!contig && (ntiles + 7) / 8 > 65535) return TRID_ERR_UNSUPPORTED;  // grid.y limit
-    // the kernels' 32-bit thread and line indices
-    if (L.nsys * ntiles >= (int64_t(1) << 31) || L.nsys >= (int64_t(1) << 31))
-        return TRID_ERR_UNSUPPORTED;
-    if (ws_bytes < long_ws_bytes<T>(L.nsys, L.n) || ws == nullptr) return TRID_ERR_ALLOC;
-    // FP64 up to 4096 rows, FP32 up to 8192: one pass (it needs no scratch, but is
-    // taken only where the passes could run, so that the same calls succeed)
+    // FP64 up to 4096 rows, FP32 up to 8192: one pass
     if (launch_team<T>(a, b, c, d, out, acc, L, st)) return TRID_OK;
     T *ra = reinterpret_cast<T *>(ws);
     T *rc = reinterpret_cast<T *>(ws + one);
