@@ -1,15 +1,16 @@
 """Strided systems longer than 256 rows (y/z axes), FP32: the cluster path
-(one CTA per chunk of 256 rows, the chunks' responses to the unknowns outside
-them joined by a chunk-level solve across the cluster) for up to 16 chunks,
-and the multi-pass path beyond.  Whole meshes against the FP64 oracle,
-element by element: chunk counts 2..16 (clusters of 2, 3, 4, 5, 8, 12, 16)
-and 17, 36, ragged last chunks of 1, 255 and 4 rows, mesh widths that leave
-partial 16-wide strips, several outer slices, accumulate mode, the unread a
-of first rows and c of last rows poisoned with NaN.  GPU only."""
+(one CTA per chunk of 256 rows, 512 above 2048, the chunks' responses to the
+unknowns outside them joined by a chunk-level solve across the cluster) for up
+to 4096 rows, the block per few systems that takes up to 1024 rows when there
+are few of them, and the passes beyond.  Whole meshes against the FP64 oracle,
+element by element: ragged last chunks of 1, 255 and 4 rows, mesh widths that
+leave partial 16-wide strips, several outer slices, accumulate mode, the unread
+a of first rows and c of last rows poisoned with NaN.  GPU only."""
 import numpy as np
 import pytest
 
 import oracle
+from graphs import graph_text
 from paper_2201_03950_gb300 import inputs, trid
 
 torch = pytest.importorskip("torch")
@@ -65,6 +66,45 @@ def test_accumulate(dims, k):
     assert torch.equal(td, d0)
     got = tu.cpu().numpy().astype(np.float64) - u0.astype(np.float64)
     assert normwise(got, ref) <= TOL
+
+
+def many(n):
+    """Systems of n rows enough for clusters: more than two strips of 16 per SM."""
+    return 16 * (2 * torch.cuda.get_device_properties(0).multi_processor_count + 1) + 4
+
+
+@pytest.mark.parametrize("n", [257, 300, 512, 513, 767, 768])
+@pytest.mark.parametrize("acc", [False, True], ids=["store", "acc"])
+@pytest.mark.filterwarnings("ignore:DEBUG")
+def test_clusters_of_two_and_three(n, acc, tmp_path):
+    dims = (many(n), n)
+    total = dims[0] * n
+    a, b, c, d = inputs.dominant_system((total,), seed=n, dtype=np.float32)
+    ref = oracle.solve_mesh(a, b, c, d, dims, 1)
+    ta, tb, tc, td = (torch.from_numpy(v).cuda() for v in (a, b, c, d))
+    poison(ta, tc, dims, 1)
+    u = torch.zeros_like(td) if acc else None
+    x = td.clone()
+    got = trid.solve(ta, tb, tc, x, dims, 1, u=u)
+    assert normwise(got.cpu().numpy(), ref) <= TOL
+    assert "k_chunk_cluster" in graph_text(lambda: trid.solve(ta, tb, tc, x, dims, 1, u=u),
+                                           tmp_path / "graph.dot")
+
+
+@pytest.mark.parametrize("dims", [(8192, 512), (3000, 1400), (4096, 2048), (4096, 4096)])
+def test_stored_many_strips_repeated(dims):
+    """Several strips of systems per cluster, stored, twenty times from inputs that
+    stay in the L2 cache (the smaller ones): the copy of a strip must not overtake
+    the reads of the strip before it."""
+    n = int(np.prod(dims))
+    a, b, c, d = inputs.dominant_system((n,), seed=11, dtype=np.float32)
+    ta, tb, tc, td = (torch.from_numpy(v).cuda() for v in (a, b, c, d))
+    ref = torch.from_numpy(oracle.solve_mesh(a, b, c, d, dims, 1)).cuda()
+    scale = ref.abs().max()
+    x = torch.empty_like(td)
+    for _ in range(20):
+        trid.solve(ta, tb, tc, x.copy_(td), dims, 1)
+        assert ((x - ref).abs().max() / scale).item() <= TOL
 
 
 def test_weak_dominance():

@@ -1,9 +1,9 @@
-"""Contiguous systems of 256 < N <= 4096 rows (FP32), the bulk-copy staged
-one-pass kernel: every team width (N <= 512, 1024, 2048, 4096), lengths just
-above and below each width, batches that end in a partial stage, accumulate
-and in-place modes, the unit-diagonal reduced systems of longer systems, and
-unaligned arrays (served by the multi-pass path).  Whole meshes against the
-FP64 oracle, element by element.  GPU only."""
+"""Contiguous systems of 256 < N <= 4096 rows (FP32): the bulk-copy staged
+one-pass kernel above 512 rows with every team width (N <= 1024, 2048, 4096), one
+warp per system up to 512, lengths just above and below each, batches that end
+in a partial stage, accumulate and in-place modes, the unit-diagonal reduced
+systems of longer systems, and unaligned arrays (one block per few systems).
+Whole meshes against the FP64 oracle, element by element.  GPU only."""
 import numpy as np
 import pytest
 
@@ -27,7 +27,8 @@ def system(n, nsys, seed):
     return a, b, c, d
 
 
-CASES = [(260, 1), (260, 9), (264, 300), (508, 17), (512, 64), (516, 5), (1020, 3), (1024, 33),
+CASES = [(260, 1), (260, 9), (264, 300), (508, 17), (512, 64), (516, 1), (516, 5), (516, 9), (520, 300),
+         (764, 17), (768, 64), (1020, 3), (1024, 33),
          (1028, 7), (2044, 2), (2048, 11), (2052, 3), (4092, 5), (4096, 1), (4096, 40)]
 
 
@@ -45,7 +46,7 @@ def test_against_oracle(n, nsys):
     assert normwise(td.cpu().numpy(), ref) <= TOL
 
 
-@pytest.mark.parametrize("n,nsys", [(264, 13), (1024, 6), (4096, 3)], ids=str)
+@pytest.mark.parametrize("n,nsys", [(264, 13), (516, 13), (1024, 6), (4096, 3)], ids=str)
 def test_accumulate(n, nsys):
     a, b, c, d = system(n, nsys, seed=3)
     dims = (n, nsys)
@@ -74,9 +75,9 @@ def test_longer_systems_reduce_into_it(n):
     assert normwise(td.cpu().numpy(), ref) <= TOL
 
 
-def test_unaligned_arrays_take_the_multipass_path():
-    """Arrays starting 4 bytes past a 16-byte boundary: same result as the
-    aligned call within rounding (different tile boundaries)."""
+def test_unaligned_arrays():
+    """Arrays starting 4 bytes past a 16-byte boundary, which bulk copies cannot
+    take (k_team): the oracle's solution too."""
     n, nsys = 1024, 9
     a, b, c, d = system(n, nsys, seed=11)
     dims = (n, nsys)
