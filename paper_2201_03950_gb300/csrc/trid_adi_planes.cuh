@@ -1,5 +1,8 @@
 // trid_adi_planes.cuh -- 3D ADI step in two passes over whole planes and whole
-// z lines (Section 4.1, Algorithm "adi"), any extents and any lambda.
+// z lines (Section 4.1, Algorithm "adi"), odd and even extents and any lambda:
+// x and y up to 160 nodes (FP64 128), the plane three times within a block's
+// shared memory (about 128 x 128 in FP32, 90 x 90 in FP64), z up to 256 (FP64 128).  The
+// launcher leaves what other schedules step faster (adi3_planes_run).
 //
 //   pass A (k_adi_planes): one block per interior z plane.  The plane and its
 //     two z neighbours are brought to shared memory; the explicit part, the x

@@ -21,8 +21,8 @@
 //  k_long_*   longer systems: tiled Thomas-PCR in passes.  k_long_reduce
 //             writes the two reduced rows of each tile to scratch, the reduced
 //             systems (2 rows per tile) are solved by a recursive call, and
-//             k_long_subst recomputes each tile and substitutes the tile-end
-//             unknowns back.
+//             k_long_subst reads each tile again and runs Thomas between its
+//             known end unknowns.
 //  k_lines_tma  contiguous FP32 systems of 512 < N <= 4096 in one pass:
 //             whole systems staged in shared memory by bulk copies, one team
 //             of warps per system (trid_lines_tma.cuh).

@@ -1,7 +1,7 @@
 """Batched ADI (adi_step_batched): every mesh of a batch against the FP64
 oracle's ADI step, for meshes resident in shared memory (all steps in one
-kernel), 3D meshes stacked through the two-pass kernels, and meshes that go
-through the single-mesh path.  GPU only."""
+kernel), 3D meshes stacked through the kernels of the 3D step, and meshes that
+go through the single-mesh path.  GPU only."""
 import numpy as np
 import pytest
 
@@ -40,8 +40,8 @@ CASES = [((32, 32), 6, 0.1, 40, np.float32), ((96, 96), 4, 0.1, 120, np.float32)
          ((200, 100), 2, 0.1, 5, np.float32), ((64, 64), 3, 0.1, 40, np.float64),
          ((32, 32, 32), 3, 0.1, 10, np.float32), ((24, 20, 16), 2, 0.15, 12, np.float32),
          ((16, 16, 16), 2, 0.1, 8, np.float64), ((5, 3, 7), 4, 0.2, 6, np.float64),
-         # larger than one block's shared memory: 3D meshes stacked along z
-         # through the two-pass kernels, or the single-mesh path
+         # larger than one block's shared memory: 3D meshes stacked along z, or
+         # the single-mesh path
          ((64, 64, 64), 2, 0.1, 3, np.float32), ((48, 32, 64), 3, 0.2, 4, np.float64),
          ((40, 40, 40), 2, 0.1, 2, np.float32), ((256, 200), 2, 0.1, 4, np.float32),
          # one 32-row tile per plane, stacked: several planes per CTA across meshes
