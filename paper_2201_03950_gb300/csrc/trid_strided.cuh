@@ -229,7 +229,6 @@ k_strided_tma(const __grid_constant__ TmaSet maps, Coef coef, T *out, Lines L, i
         }
         fence_mbar_init();
     }
-    pdl_trigger();
     pdl_wait();  // the arrays may be written by the previous kernel on the stream
     __syncthreads();
     const int64_t nxc = (L.inner + SG - 1) / SG;
@@ -239,8 +238,16 @@ k_strided_tma(const __grid_constant__ TmaSet maps, Coef coef, T *out, Lines L, i
         if (tid == NCONS) {
             const uint32_t tx = uint32_t(NSLOT) * uint32_t(n) * SG * sizeof(T);
             int k = 0;
+            // The next kernel may start when every block has come to its last batch,
+            // in short launches at once.  Blocks that started while the others still had
+            // batches to do would not be spread evenly: some SMs then hold two of
+            // the blocks with one batch more.  Along y with accumulate, a launch at
+            // once -> this: 256^3 69.5 -> 66.4 us, 1000 x 200 x 50 46.8 -> 45.7, 1000 x
+            // 100 x 50 21.5 -> 20.4; but 128^3, 3.4 batches a block, 10.8 -> 11.6.
+            const bool brief = nbatch <= 4 * int64_t(gridDim.x);
             for (int64_t bt = blockIdx.x; bt < nbatch; bt += gridDim.x, ++k) {
                 const int s = k % stages;
+                if (brief ? k == 0 : bt + gridDim.x >= nbatch) pdl_trigger();
                 if (k >= stages && !mbar_wait(&empty[s], uint32_t((k / stages) - 1) & 1u, status)) {
                     *(volatile int *)&abort_flag = 1;
                     break;
@@ -388,8 +395,8 @@ inline bool launch_strided_tma(const void *const *arrs, Coef coef, T *out, const
     const int64_t slots = int64_t(di->sm_count) * per_sm;
     const int64_t grid = nbatch < slots ? nbatch : slots;
     // programmatic dependent launch: the next direction's blocks set up while
-    // this one drains (256^3 along x, y and z 163.0 -> 160.5 us; on k_lines too
-    // it gave nothing more)
+    // this one drains (256^3 along x, y and z 163.0 -> 160.5 us, 96^3 20.6 -> 16.4, 64^3
+    // 15.6 -> 12.0; on k_lines too it gave nothing more)
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

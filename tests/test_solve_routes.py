@@ -59,19 +59,22 @@ def test_fp32_contiguous_257_to_512(acc, tmp_path):
     check((400, 1000), 0, np.float32, acc, "k_lines_chained", tmp_path)
 
 
-@pytest.mark.parametrize("n,nsys", [(260, 1), (400, 64), (512, 1000)])
-def test_chained_calls_see_each_other(n, nsys):
+@pytest.mark.parametrize("dims,k", [((260, 1), 0), ((400, 64), 0), ((512, 1000), 0), ((64, 64, 64), 1),
+                                    ((64, 64, 64), 2), ((128, 128, 128), 1), ((1000, 256, 25), 1),
+                                    ((304, 200, 90), 1)], ids=str)
+def test_chained_calls_see_each_other(dims, k):
     """Ten calls in a row, each on what the one before has written, as with a
     synchronisation in between."""
-    t = [torch.from_numpy(v).cuda() for v in inputs.dominant_system((n * nsys,), seed=n, dtype=np.float32)]
+    n = int(np.prod(dims))
+    t = [torch.from_numpy(v).cuda() for v in inputs.dominant_system((n,), seed=n, dtype=np.float32)]
     out = []
     for wait in (False, True):
         x, b, u = t[3].clone(), t[1].clone(), torch.zeros_like(t[3])
         for _ in range(10):
-            trid.solve(t[0], b, t[2], x, (n, nsys), 0)
+            trid.solve(t[0], b, t[2], x, dims, k)
             if wait:
                 torch.cuda.synchronize()
-            trid.solve(t[0], b, t[2], x, (n, nsys), 0, u=u)
+            trid.solve(t[0], b, t[2], x, dims, k, u=u)
             if wait:
                 torch.cuda.synchronize()
             torch.add(t[1], u.abs(), out=b)     # the next call's coefficients
