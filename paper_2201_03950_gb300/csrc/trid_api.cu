@@ -79,7 +79,7 @@ using LaunchCache = std::unordered_map<LaunchKey, int, LaunchKeyHash>;
 constexpr size_t kLaunchCacheMax = 1 << 16;
 LaunchCache g_occ;      // blocks per SM (csize 0)
 LaunchCache g_ccache;   // resident clusters
-LaunchCache g_limit;    // dynamic shared memory allowed (threads, csize, smem 0)
+LaunchCache g_limit;    // dynamic shared memory allowed (csize, threads, smem 0)
 
 bool launch_find(const LaunchCache &c, const LaunchKey &k, int &v) {
     const auto it = c.find(k);
@@ -99,25 +99,27 @@ void launch_forget(LaunchCache &c, int dev) {
         it = it->first.dev == dev ? c.erase(it) : std::next(it);
 }
 
-// The dynamic shared memory that launches of `kernel` may ask for.  The limit is
-// an attribute of the function, shared by every thread of the process: it is
-// raised once, to all that a block can have, so that no query for a small size
-// takes it away between another thread's query and launch.
-bool raise_smem_limit(const void *kernel, int dev, int max_optin, int &limit) {
-    const LaunchKey key{kernel, dev, 0, 0, 0};
-    if (launch_find(g_limit, key, limit)) return true;
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-    if (e == cudaSuccess) {
-        limit = max_optin - int(fa.sharedSizeBytes);
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+// Lets launches of `kernel` ask for `smem` bytes of dynamic shared memory.  The
+// limit is an attribute of the function, shared by every thread of the process:
+// it is only ever raised, from the largest size asked for so far, whether or not
+// that query is still kept, so that no query for a small size takes it away
+// between another thread's query and launch.
+bool raise_smem_limit(const void *kernel, int dev, int smem) {
+    int *raised = nullptr;
+    try {
+        raised = &g_limit.emplace(LaunchKey{kernel, dev, 0, 0, 0}, 0).first->second;
+    } catch (...) {   // no memory
+        return false;
     }
+    if (*raised >= smem) return true;
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) {
         cudaGetLastError();
         note_cuda_error(e);
         return false;
     }
-    launch_keep(g_limit, key, limit);
+    *raised = smem;
     return true;
 }
 }  // namespace
@@ -160,17 +162,14 @@ int cluster_capacity(const void *kernel, int csize, int threads, size_t smem) {
 
 int kernel_blocks_per_sm(const void *kernel, int threads, size_t smem) {
     int dev = 0;
-    const DeviceInfo *di = device_info();
-    if (!di || cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lk(g_pool_mu);
     const LaunchKey key{kernel, dev, 0, threads, smem};
-    int blocks = 0, limit = 0;
+    int blocks = 0;
     if (launch_find(g_occ, key, blocks)) return blocks;
-    if (!raise_smem_limit(kernel, dev, di->max_smem_optin, limit)) return 0;
+    if (!raise_smem_limit(kernel, dev, int(smem))) return 0;
     const cudaError_t oe =
-        smem > size_t(limit) ? cudaErrorInvalidValue
-                             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel,
-                                                                             threads, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, threads, smem);
     if (oe != cudaSuccess) {
         cudaGetLastError();
         note_cuda_error(oe);

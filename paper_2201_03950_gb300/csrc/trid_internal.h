@@ -52,9 +52,8 @@ int cluster_capacity(const void *kernel, int csize, int threads, size_t smem);
 
 // Blocks of `kernel` resident per SM for (threads, dynamic smem) on the
 // current device, after raising the kernel's dynamic shared-memory limit to
-// the most a block can have (once per kernel and device).  Both results are
-// kept, so a launch in a time-stepping loop costs no extra driver calls.  0 on
-// failure.
+// `smem` (it is never lowered).  Both results are kept, so a launch in a
+// time-stepping loop costs no extra driver calls.  0 on failure.
 int kernel_blocks_per_sm(const void *kernel, int threads, size_t smem);
 
 // Batched solve with caller-chosen scratch (checks arguments on the host;
