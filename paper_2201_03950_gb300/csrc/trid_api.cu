@@ -8,8 +8,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <iterator>
+#include <map>
 #include <mutex>
-#include <unordered_map>
+#include <utility>
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -55,49 +56,51 @@ const DeviceInfo *device_info() {
 namespace {
 // Results of the launch queries, kept per (kernel, device, cluster size, threads,
 // dynamic shared memory).  Several kernels' shared memory follows the extents, so
-// a process that meets many sizes asks many keys: a hash table, emptied if it
-// ever holds kLaunchCacheMax.
-struct LaunchKey {
-    const void *kernel;
-    int dev, csize, threads;
-    size_t smem;
-    bool operator==(const LaunchKey &o) const {
-        return kernel == o.kernel && dev == o.dev && csize == o.csize && threads == o.threads &&
-               smem == o.smem;
-    }
-};
-struct LaunchKeyHash {
-    size_t operator()(const LaunchKey &k) const {
-        uint64_t h = uint64_t(reinterpret_cast<uintptr_t>(k.kernel));
-        const uint64_t rest[2] = {uint64_t(k.dev) << 40 | uint64_t(k.csize) << 20 |
-                                      uint64_t(k.threads), uint64_t(k.smem)};
-        for (uint64_t v : rest) h = (h ^ v) * 0x9e3779b97f4a7c15ull, h ^= h >> 29;
-        return size_t(h);
-    }
-};
-using LaunchCache = std::unordered_map<LaunchKey, int, LaunchKeyHash>;
-constexpr size_t kLaunchCacheMax = 1 << 16;
-LaunchCache g_occ;      // blocks per SM (csize 0)
-LaunchCache g_ccache;   // resident clusters
-LaunchCache g_limit;    // dynamic shared memory allowed (csize, threads, smem 0)
+// a process that meets many sizes asks many keys: a hash table with the entries in
+// place (a lookup is mostly one cache line, 2.9 us for a call as with a few entries
+// in a list), emptied when it has filled up to three quarters.
+struct LaunchTable {
+    static constexpr unsigned SIZE = 4096;
+    struct Entry {
+        const void *kernel;   // nullptr: empty
+        uint64_t shape;
+        int value;
+    };
+    Entry e[SIZE];
+    unsigned used;
 
-bool launch_find(const LaunchCache &c, const LaunchKey &k, int &v) {
-    const auto it = c.find(k);
-    if (it == c.end()) return false;
-    v = it->second;
-    return true;
-}
-void launch_keep(LaunchCache &c, const LaunchKey &k, int v) {
-    try {
-        if (c.size() >= kLaunchCacheMax) c.clear();
-        c.emplace(k, v);
-    } catch (...) {   // no memory: asked again next time
+    static uint64_t shape_of(int dev, int csize, int threads, size_t smem) {
+        return uint64_t(dev) << 58 | uint64_t(csize) << 48 | uint64_t(threads) << 32 |
+               uint64_t(uint32_t(smem));
     }
-}
-void launch_forget(LaunchCache &c, int dev) {
-    for (auto it = c.begin(); it != c.end();)
-        it = it->first.dev == dev ? c.erase(it) : std::next(it);
-}
+    // The key's entry, or the empty one where it belongs.
+    Entry *at(const void *kernel, uint64_t shape) {
+        const uint64_t h = (uint64_t(reinterpret_cast<uintptr_t>(kernel)) ^
+                            shape * 0x9e3779b97f4a7c15ull) * 0xff51afd7ed558ccdull;
+        unsigned i = unsigned(h >> 40) % SIZE;
+        while (e[i].kernel && (e[i].kernel != kernel || e[i].shape != shape)) i = (i + 1) % SIZE;
+        return &e[i];
+    }
+    bool find(const void *kernel, uint64_t shape, int &value) {
+        const Entry *x = at(kernel, shape);
+        if (!x->kernel) return false;
+        value = x->value;
+        return true;
+    }
+    void keep(const void *kernel, uint64_t shape, int value) {
+        if (used >= SIZE / 4 * 3) clear();
+        Entry *x = at(kernel, shape);
+        if (!x->kernel) ++used;
+        *x = Entry{kernel, shape, value};
+    }
+    void clear() {
+        std::memset(static_cast<void *>(e), 0, sizeof(e));
+        used = 0;
+    }
+};
+LaunchTable g_occ;      // blocks per SM (cluster size 0)
+LaunchTable g_ccache;   // resident clusters
+std::map<std::pair<const void *, int>, int> g_limit;   // (kernel, device): shared memory allowed
 
 // Lets launches of `kernel` ask for `smem` bytes of dynamic shared memory.  The
 // limit is an attribute of the function, shared by every thread of the process:
@@ -107,7 +110,7 @@ void launch_forget(LaunchCache &c, int dev) {
 bool raise_smem_limit(const void *kernel, int dev, int smem) {
     int *raised = nullptr;
     try {
-        raised = &g_limit.emplace(LaunchKey{kernel, dev, 0, 0, 0}, 0).first->second;
+        raised = &g_limit.emplace(std::make_pair(kernel, dev), 0).first->second;
     } catch (...) {   // no memory
         return false;
     }
@@ -128,9 +131,9 @@ int cluster_capacity(const void *kernel, int csize, int threads, size_t smem) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    const LaunchKey key{kernel, dev, csize, threads, smem};
+    const uint64_t shape = LaunchTable::shape_of(dev, csize, threads, smem);
     int n = 0;
-    if (launch_find(g_ccache, key, n)) return n;
+    if (g_ccache.find(kernel, shape, n)) return n;
     if (csize > 8) {
         const cudaError_t ae =
             cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -156,7 +159,7 @@ int cluster_capacity(const void *kernel, int csize, int threads, size_t smem) {
         cudaGetLastError();
         n = 0;
     }
-    launch_keep(g_ccache, key, n);
+    g_ccache.keep(kernel, shape, n);
     return n;
 }
 
@@ -164,9 +167,9 @@ int kernel_blocks_per_sm(const void *kernel, int threads, size_t smem) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    const LaunchKey key{kernel, dev, 0, threads, smem};
+    const uint64_t shape = LaunchTable::shape_of(dev, 0, threads, smem);
     int blocks = 0;
-    if (launch_find(g_occ, key, blocks)) return blocks;
+    if (g_occ.find(kernel, shape, blocks)) return blocks;
     if (!raise_smem_limit(kernel, dev, int(smem))) return 0;
     const cudaError_t oe =
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, threads, smem);
@@ -175,7 +178,7 @@ int kernel_blocks_per_sm(const void *kernel, int threads, size_t smem) {
         note_cuda_error(oe);
         return 0;
     }
-    launch_keep(g_occ, key, blocks);
+    g_occ.keep(kernel, shape, blocks);
     return blocks;
 }
 
@@ -278,9 +281,10 @@ static void forget_device(int dev) {
     g_info_ok[dev] = false;
     if (g_aux_stream[dev]) cudaStreamDestroy(g_aux_stream[dev]);
     g_aux_stream[dev] = nullptr;
-    launch_forget(g_occ, dev);
-    launch_forget(g_ccache, dev);
-    launch_forget(g_limit, dev);
+    g_occ.clear();
+    g_ccache.clear();
+    for (auto it = g_limit.begin(); it != g_limit.end();)
+        it = it->first.second == dev ? g_limit.erase(it) : std::next(it);
 }
 
 cudaStream_t aux_stream() {
