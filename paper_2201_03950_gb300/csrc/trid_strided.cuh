@@ -229,6 +229,14 @@ k_strided_tma(const __grid_constant__ TmaSet maps, Coef coef, T *out, Lines L, i
         }
         fence_mbar_init();
     }
+    // The next kernel may start when every block has come to its last batch (below),
+    // in short launches at once.  Blocks that started while the others still had
+    // batches to do would not be spread evenly: some SMs then hold two of the blocks
+    // with one batch more.  Along y with accumulate, all launches at once -> this:
+    // 256^3 69.5 -> 66.4 us, 1000 x 200 x 50 46.8 -> 45.7, 1000 x 100 x 50 21.5 -> 20.4;
+    // but 128^3, 3.4 batches a block, 10.8 -> 11.6.
+    const bool brief = nbatch <= 4 * int64_t(gridDim.x);
+    if (brief) pdl_trigger();
     pdl_wait();  // the arrays may be written by the previous kernel on the stream
     __syncthreads();
     const int64_t nxc = (L.inner + SG - 1) / SG;
@@ -238,16 +246,9 @@ k_strided_tma(const __grid_constant__ TmaSet maps, Coef coef, T *out, Lines L, i
         if (tid == NCONS) {
             const uint32_t tx = uint32_t(NSLOT) * uint32_t(n) * SG * sizeof(T);
             int k = 0;
-            // The next kernel may start when every block has come to its last batch,
-            // in short launches at once.  Blocks that started while the others still had
-            // batches to do would not be spread evenly: some SMs then hold two of
-            // the blocks with one batch more.  Along y with accumulate, a launch at
-            // once -> this: 256^3 69.5 -> 66.4 us, 1000 x 200 x 50 46.8 -> 45.7, 1000 x
-            // 100 x 50 21.5 -> 20.4; but 128^3, 3.4 batches a block, 10.8 -> 11.6.
-            const bool brief = nbatch <= 4 * int64_t(gridDim.x);
             for (int64_t bt = blockIdx.x; bt < nbatch; bt += gridDim.x, ++k) {
                 const int s = k % stages;
-                if (brief ? k == 0 : bt + gridDim.x >= nbatch) pdl_trigger();
+                if (!brief && bt + gridDim.x >= nbatch) pdl_trigger();
                 if (k >= stages && !mbar_wait(&empty[s], uint32_t((k / stages) - 1) & 1u, status)) {
                     *(volatile int *)&abort_flag = 1;
                     break;
