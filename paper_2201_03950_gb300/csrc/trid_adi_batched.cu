@@ -6,12 +6,12 @@
 // 2D meshes that fit one block's shared memory, up to 160 (FP64: 128) nodes
 // along an axis, run every step of the call on chip in k_adi_plane
 // (trid_adi_plane.cuh).  Small 3D meshes (and the 2D ones beyond that, or in FP64
-// mostly padding there) do so in k_adi_fused: a block loads the mesh once, runs all nsteps steps in
-// shared memory and writes it back: per step the 5-point / 7-point RHS, then
-// one thread per line runs the Thomas sweeps of each axis with the constant
-// operator's pivots factored once on the host, the last axis adding its result
-// into u.  Rows are padded to an odd stride, so the threads of a warp (one line
-// each) hit distinct banks on every axis.  The other 3D meshes, and in FP32 most of
+// mostly padding there) do so in k_adi_fused: a block loads the mesh once, runs
+// all nsteps steps in shared memory and writes it back: per step the 5-point /
+// 7-point RHS, then one thread per line runs the Thomas sweeps of each axis with
+// the constant operator's pivots factored once on the host, the last axis adding
+// its result into u.  Rows are padded to an odd stride, so the threads of a warp
+// (one line each) hit distinct banks on every axis.  The other 3D meshes, and in FP32 most of
 // the small ones, run stacked along z (each mesh keeps its own boundary planes)
 // through the windowed kernels where those take them, else the whole-plane ones,
 // and with extents that are multiples of 16 (z from 32) the two-pass ones; those

@@ -636,9 +636,11 @@ static bool launch_chunk_cluster(const T *a, const T *b, const T *c, const T *d,
 // 256, 41 / 45); contiguous ones, whose rounds are shorter, at about 6000 (256 rows: 68
 // against 66 us there, 70 against 78 at 7400; 192 rows 53 against 65).  At 65536
 // systems of 256 rows they are 305 against 655 us (strided) and 381 against 596 us
-// (contiguous).  Accumulating, d' fills the shared memory too: beyond 232 rows an SM
-// holds three warps, and a round of 48 systems per SM takes 1.27 rounds of the tiled
-// kernel (7400 systems of 256 rows 119 against 94 us, 15000 180 / 170).
+// (contiguous).  Accumulating, d' fills the shared memory too, beyond 232 rows an SM
+// holds three warps, and just above 48 systems per SM the tiled kernel would be
+// faster (7400 systems of 256 rows 119 against 94 us, 9800 121 / 120); strided systems
+// come here all the same, so that storing and accumulating give the same bits
+// (the differentiable ADI recomputes with the one what it did with the other).
 // Contiguous systems only when their halves are whole 32-byte vectors (with
 // scalar loads 378 us against 402 us at 43571 systems of 201 rows, and slower
 // than that at two warps per block), and not when accumulating (d' then
@@ -674,11 +676,6 @@ static bool launch_twist(const T *a, const T *b, const T *c, const T *d, T *out,
         }
         const bool early = L.n <= 24 || (L.n > 128 && L.n <= 192);
         if (L.nsys <= (early ? 30 : 32) * sms) return false;
-        if (acc) {
-            const int64_t warps = di->smem_per_sm / (twist_smem(int(L.n), false, true, 1) + 1024);
-            const int64_t rounds = (L.nsys - 1) / (TW_SYS * (warps > 0 ? warps : 1) * sms) + 1;
-            if (warps < 4 && 14 * rounds > 10 * ((L.nsys - 1) / (32 * sms) + 1)) return false;
-        }
         return acc ? launch_twist_form<true, false, 1>(a, b, c, d, out, L, st)
                    : launch_twist_form<false, false, 1>(a, b, c, d, out, L, st);
     }

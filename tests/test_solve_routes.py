@@ -45,15 +45,6 @@ def test_fp64_short_strided_early(n, tmp_path):
     check((30 * sms + 4, n), 1, np.float64, False, "k_twist", tmp_path)
 
 
-def test_fp64_accumulating_rounds(tmp_path):
-    """256 rows: a round of 48 systems per SM against rounds of 32."""
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
-    check((48 * sms + 4, 256), 1, np.float64, True, "k_strided", tmp_path)
-    check((48 * sms + 4, 256), 1, np.float64, False, "k_twist", tmp_path)
-    check((48 * sms + 4, 200), 1, np.float64, True, "k_twist", tmp_path)
-    check((64 * sms + 4, 256), 1, np.float64, True, "k_twist", tmp_path)
-
-
 @pytest.mark.parametrize("acc", [False, True], ids=["store", "acc"])
 def test_fp32_contiguous_257_to_512(acc, tmp_path):
     check((400, 1000), 0, np.float32, acc, "k_lines_chained", tmp_path)

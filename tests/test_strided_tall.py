@@ -44,7 +44,8 @@ def test_system_counts(nsys, n, acc):
 
 
 @pytest.mark.parametrize("dims", [(1000, 300), (1024, 700), (1024, 1000), (2048, 900), (4864, 512),
-                                  (5000, 600), (37, 800), (1001, 1001), (4700, 200)])
+                                  (5000, 600), (37, 800), (1001, 1001), (4700, 200), (4865, 256),
+                                  (7400, 250), (9800, 256), (4800, 100)])
 def test_stored_and_accumulated_bits_agree(dims):
     """The differentiable ADI recomputes with stored solves what its forward
     accumulated (u = 0 + x), also into an array of another alignment."""
